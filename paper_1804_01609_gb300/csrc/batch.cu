@@ -25,6 +25,7 @@
 #include "common.cuh"
 #include "device_ops.cuh"
 #include "kernels.cuh"
+#include "reduced.cuh"
 
 namespace rbfsl {
 
@@ -81,16 +82,16 @@ __global__ void batch_trace_kernel(const BatchDesc *__restrict__ d, int np, int6
                         Xi[3 * j + 2]);
 }
 
-// Shared memory of one point. Direct mode: system region (ldl_doubles), then the stencil (n
+// Shared memory of one point. Direct mode: system region (weights_doubles), then the stencil (n
 // int). Centre mode: right-hand side and solution (2 m double). The k-NN buffers (cap double +
 // cap int + 1 int) alias the start of the region: the search ends, and its result is copied
 // out, before the system or the right-hand side is written. A 109 x 109 system then takes
 // 55.6 KB, four points per SM.
-__host__ __device__ inline int batch_region_doubles(int mode, int n, int m, int ld) {
-    return mode == RBFSL_DIRECT ? ldl_doubles(n, m) + (n + 1) / 2 : 2 * m;
+__host__ __device__ inline int batch_region_doubles(int mode, int n, int m, int ell, int half) {
+    return mode == RBFSL_DIRECT ? weights_doubles(n, m, ell, half) + (n + 1) / 2 : 2 * m;
 }
-__host__ __device__ inline int batch_point_doubles(int mode, int n, int m, int ld, int cap) {
-    const int region = batch_region_doubles(mode, n, m, ld), knn = cap + (cap + 2) / 2;
+__host__ __device__ inline int batch_point_doubles(int mode, int n, int m, int ell, int half, int cap) {
+    const int region = batch_region_doubles(mode, n, m, ell, half), knn = cap + (cap + 2) / 2;
     return region > knn ? region : knn;
 }
 
@@ -130,8 +131,8 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
         const int p = p_begin + find_problem(d + p_begin, np, tile, true);
         const BatchDesc &b = d[p];
         if (!b.active) continue;
-        const int n = b.n, m = b.m, ld = b.ld, cap = knn_cap(b.mode == RBFSL_DIRECT ? n : 1);
-        const int per = batch_point_doubles(b.mode, n, m, ld, cap);
+        const int n = b.n, m = b.m, cap = knn_cap(b.mode == RBFSL_DIRECT ? n : 1);
+        const int per = batch_point_doubles(b.mode, n, m, b.ell, b.half, cap);
         const int k = b.mode == RBFSL_DIRECT ? n : 1;
         if (b.ppt == 4 || b.mode == RBFSL_CENTER) {
             // one warp per point
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
             if (i >= b.N) continue;
             double *base = sm + (size_t)warp * per;
             double *A = base;
-            int32_t *S = reinterpret_cast<int32_t *>(base + ldl_doubles(n, m));  // direct only
+            int32_t *S = reinterpret_cast<int32_t *>(base + weights_doubles(n, m, b.ell, b.half));  // direct only
             double *bd = base;  // aliases the region (see batch_point_doubles)
             int *bi = reinterpret_cast<int *>(bd + cap);
             int *cnt = bi + cap;
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
                 for (int j = lane; j < n; j += 32) S[j] = bi[j];
                 __syncwarp();
                 double *wv = nullptr;
-                rc = weights_point_ldl<1>(A, b.X, S, n, m, b.ell, b.half, px, py, pz, lane, wv);
+                rc = weights_point<1>(A, b.X, S, n, m, b.ell, b.half, px, py, pz, lane, wv);
                 if (rc == RBFSL_OK) batch_gather(b, wv, S, i, lane);
             } else {
                 const int64_t kc = bi[0];
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
             // four warps per point (direct mode)
             const int64_t i = tile - b.tile0;
             double *A = sm;
-            int32_t *S = reinterpret_cast<int32_t *>(sm + ldl_doubles(n, m));
+            int32_t *S = reinterpret_cast<int32_t *>(sm + weights_doubles(n, m, b.ell, b.half));
             double *bd = sm;  // aliases the region (see batch_point_doubles)
             int *bi = reinterpret_cast<int *>(bd + cap);
             int *cnt = bi + cap;
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
             }
             __syncthreads();
             double *wv = nullptr;
-            const int rc = weights_point_ldl<4>(A, b.X, S, n, m, b.ell, b.half, px, py, pz, t, wv);
+            const int rc = weights_point<4>(A, b.X, S, n, m, b.ell, b.half, px, py, pz, t, wv);
             if (warp == 0) {
                 if (rc == RBFSL_OK) {
                     batch_gather(b, wv, S, i, lane);
@@ -279,7 +280,7 @@ int default_ppt(const rbfsl_batch *b, int n, int ell, int mode) {
     auto it = b->tile_rule.find(class_key(n, ell));
     if (it != b->tile_rule.end()) return it->second;
     const int m = n + (ell + 1) * (ell + 1);
-    return ldl_doubles(n, m) * 8 > kWeightsSmallBytes ? 1 : 4;  // the single-problem rule
+    return weights_doubles(n, m, ell, 0) * 8 > kWeightsSmallBytes ? 1 : 4;  // the single-problem rule
 }
 
 void free_problem(HostProblem &h) {
@@ -323,7 +324,7 @@ int rebuild(rbfsl_batch *b) {
             nodes += d.N;
             tiles += d.ppt == 4 ? (d.N + 3) / 4 : d.N;
             const int cap = knn_cap(d.mode == RBFSL_DIRECT ? d.n : 1);
-            const int per = batch_point_doubles(d.mode, d.n, d.m, d.ld, cap) * 8;
+            const int per = batch_point_doubles(d.mode, d.n, d.m, d.ell, d.half, cap) * 8;
             cl.smem = std::max(cl.smem, d.ppt == 4 ? 4 * per : per);
             b->slot_of[id] = (int)tab.size();
             tab.push_back(d);
@@ -690,7 +691,7 @@ int rbfsl_batch_autotune(rbfsl_batch *b, int *choices, int max_choices) {
         float best_ms = 1e30f;
         int best = 1;
         const int kn = (int)(key / 64), kell = (int)(key % 64), km = kn + (kell + 1) * (kell + 1);
-        const int per_bytes = batch_point_doubles(RBFSL_DIRECT, kn, km, (km + 1) | 1, knn_cap(kn)) * 8;
+        const int per_bytes = batch_point_doubles(RBFSL_DIRECT, kn, km, kell, 0, knn_cap(kn)) * 8;
         for (int ppt : {4, 1}) {
             if (ppt == 4 && 4 * per_bytes > max_smem) continue;
             // only this class active, with the candidate tile shape

@@ -1,18 +1,20 @@
 // Stencil weights of the augmented local RBF interpolant (Sec. 2.2, Eqs. rbf_poly and
 // rbf_poly_linsys), FP64 throughout.
 //
-// Each point's group of warps assembles the lower triangle of the symmetric (n + M) x (n + M)
-// saddle-point system in shared memory (M = (ell+1)^2):
-//     [ A    P ] w~ = [ phi(|p - x_j|) ]      A_jk = |x_j - x_k|^pw   (PHS, zero diagonal)
-//     [ P^T  0 ]      [ Y(p)           ]      P_jc = Y_c(x_j)
-// and solves it by a blocked Bunch-Kaufman L D L^T factorisation (weights_point_ldl: panels of
-// four pivot columns updated on the fly, one trailing update per panel): ~m^3 / 3 flops per
-// point, half of Gaussian elimination's, bound by GB300's FP64 rate. Small systems take one warp
-// per point (four points per block); larger ones four warps per point, several points per SM so
-// that one point's pivot steps overlap the others' trailing updates.
+// The weights w solve the symmetric (n + M) x (n + M) saddle-point system (M = (ell+1)^2)
+//     [ A    P ] [ w      ]   [ phi(|p - x_j|) ]      A_jk = |x_j - x_k|^pw   (PHS, zero diagonal)
+//     [ P^T  0 ] [ lambda ] = [ Y(p)           ]      P_jc = Y_c(x_j)
+// Each point's group of warps solves it in shared memory, reduced to the null space of P^T
+// (reduced.cuh) or, for exponents above the harmonics' order and n <= M, as a whole by a blocked
+// Bunch-Kaufman L D L^T (weights_point_ldl): ~m^3 / 3 flops per point either way (m = n + M), bound
+// by GB300's FP64 rate. Small systems take one warp per point (four points per block); larger ones
+// four warps per point, several points per SM so that one point's serial steps overlap the others'
+// products. N = 40,962, reduced form against the indefinite factorisation: m = 109 24.4 ms against
+// 30.3 ms, m = 71 7.8 ms against 10.1 ms, m = 40 2.3 ms against 2.9 ms.
 #include "common.cuh"
 #include "kernels.cuh"
 #include "device_ops.cuh"
+#include "reduced.cuh"
 
 namespace rbfsl {
 
@@ -77,7 +79,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32, 7) weights_kernel(Wei
     if (i >= a.Nq) return;  // NW == 1 only (with NW > 1 the grid has exactly Nq blocks)
     double *R = smem + (size_t)g * a.region_doubles;
     double *w = nullptr;
-    const int rc = weights_point_ldl<NW>(R, a.X, a.idx + i * a.n, a.n, a.m, a.ell, a.half,
+    const int rc = weights_point<NW>(R, a.X, a.idx + i * a.n, a.n, a.m, a.ell, a.half,
                                          a.P[3 * i], a.P[3 * i + 1], a.P[3 * i + 2], t, w);
     if (t >= kWarp) return;
     const int n = a.n, lane = t;
@@ -114,7 +116,7 @@ int launch_weights(const double *x, const int32_t *idx, int64_t Nq, int n, int e
     a.X = x; a.idx = idx; a.Nq = Nq; a.n = n; a.ell = ell; a.half = (power - 1) / 2;
     a.P = p; a.status = status;
     a.m = n + (ell + 1) * (ell + 1);
-    a.region_doubles = ldl_doubles(n, a.m);
+    a.region_doubles = weights_doubles(n, a.m, ell, a.half);
     const int bytes = a.region_doubles * 8;
     if (bytes > kWeightsSmallBytes) {
         // larger systems (m >~ 45): four warps per point (one per SM sub-partition), one point

@@ -1,0 +1,50 @@
+"""Stencil weights in the reduced (null-space) form at the edges of its launch shapes and panels,
+and the systems that take the pivoted factorisation instead."""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1804_01609_gb300 import inputs, rbfsl  # noqa: E402
+
+import test_gpu_local as loc  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+# K = n - M of 1, 7, 8, 9, 16 (panels of 8); n + 1 of 32 and 33 (a warp of points); one harmonic
+# (K up to 158), 64 harmonics, the largest systems; one and four warps per point; and exponents
+# above the harmonics' order (p = 9, ell = 2) and n < M, which keep the indefinite factorisation
+@pytest.mark.parametrize("n,ell,p", [(10, 2, 5), (16, 2, 5), (17, 2, 3), (18, 2, 5), (32, 3, 7), (31, 2, 5), (32, 2, 5),
+                                     (9, 0, 1), (159, 0, 1), (135, 4, 9), (96, 7, 15), (84, 4, 9), (55, 3, 7),
+                                     (84, 4, 3), (31, 2, 9)])
+def test_reduced_weights_interpolate(orc, n, ell, p):
+    N = 1200
+    X = inputs.nodes(N, 5)
+    P = loc._departures(X, 6)[:301]
+    I = orc.knn(X, P, n)
+    w = torch.empty((len(P), n), dtype=torch.float64, device="cuda")
+    st = torch.empty(len(P), dtype=torch.int32, device="cuda")
+    rbfsl.rbfsl_stencil_weights(loc._t(X), loc._t(I, torch.int32), n, ell, rbfsl.PHS, p, loc._t(P), w, st)
+    assert (st.cpu().numpy() == 0).all()
+    W = w.cpu().numpy()
+    q = inputs.config_local_deformation(N=N, n_random=4).tracers(X)
+    loc.assert_within_noise_floor(orc, X, I, P, q, np.einsum("ij,ijt->it", W, q[I]), ell, p)
+
+
+def test_rank_deficient_harmonics_are_singular():
+    """Nodes on the equator: the harmonic proportional to z vanishes at all of them, P has a zero
+    column and the system is exactly singular, as by the indefinite factorisation."""
+    n = 12
+    a = 2.0 * math.pi * np.arange(40) / 40
+    X = np.stack([np.cos(a), np.sin(a), np.zeros_like(a)], axis=1)
+    b = a[:7] + 0.03
+    P = np.stack([np.cos(b), np.sin(b), np.zeros_like(b)], axis=1)
+    I = np.argsort(((P[:, None] - X[None]) ** 2).sum(-1), axis=1)[:, :n]
+    w = torch.empty((len(P), n), dtype=torch.float64, device="cuda")
+    st = torch.empty(len(P), dtype=torch.int32, device="cuda")
+    rbfsl.rbfsl_stencil_weights(loc._t(X), loc._t(I, torch.int32), n, 1, rbfsl.PHS, 3, loc._t(P), w, st)
+    assert (st.cpu().numpy() == rbfsl.ESINGULAR).all()
+    assert np.isnan(w.cpu().numpy()).all()
