@@ -280,7 +280,7 @@ int default_ppt(const rbfsl_batch *b, int n, int ell, int mode) {
     auto it = b->tile_rule.find(class_key(n, ell));
     if (it != b->tile_rule.end()) return it->second;
     const int m = n + (ell + 1) * (ell + 1);
-    return weights_doubles(n, m, ell, 0) * 8 > kWeightsSmallBytes ? 1 : 4;  // the single-problem rule
+    return weights_doubles(n, m, ell, 0) * 8 > kWeightsSmallBytes || reduced_on_tensor(m - n) ? 1 : 4;  // the single-problem rule
 }
 
 void free_problem(HostProblem &h) {

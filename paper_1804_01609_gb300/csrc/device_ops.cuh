@@ -437,24 +437,26 @@ __device__ __forceinline__ long long warp_max_key(long long key) {
 }
 
 // 1 / d by Newton-Raphson iteration r <- r + r (1 - d r) (the classical reciprocal iteration,
-// each step doubling the correct bits) from an FP32 seed: the reciprocal of d's leading 24
-// significand bits (rcp.approx.f32, ~23 correct bits) with d's exponent negated, then two
-// FMA-based steps in FP64, ~1 ulp. Zero, subnormal, huge or non-finite d take the division.
+// each step doubling the correct bits): the first step in FP32 arithmetic, from rcp.approx.f32 of
+// the leading 24 significand bits and with the residual of all 53 (1 - d r formed by FMAs on the
+// two parts, its square kept), merged into an FP64 number by integer operations (~2^-46); then
+// one FP64 step, ~1 ulp. Only two of the chain's operations are on the FP64 pipe, which the other
+// points' products keep queued. Zero, subnormal, huge or non-finite d take the division.
 __device__ __forceinline__ double recip_nr(double d) {
     const long long b = __double_as_longlong(d);
     const int e = (int)((b >> 52) & 0x7ff);
     if (e < 2 || e > 2044) return 1.0 / d;
     const float mf = __int_as_float(0x3f800000 | (int)((b >> 29) & 0x7fffff));  // in [1, 2)
+    const float ml = (float)(int)(b & 0x1fffffff) * 0x1p-52f;                   // the other 29 bits
     float rf;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(mf));                     // in (0.5, 1]
+    const float tf = fmaf(-ml, rf, fmaf(-mf, rf, 1.0f));
+    const int add = __float2int_rn(rf * fmaf(tf, tf, tf) * 0x1p53f);            // in units of 2^-53
     const int fb = __float_as_int(rf);
     const long long re = (long long)(((fb >> 23) & 0xff) - 127) + 1023 - (e - 1023);
-    double r = __longlong_as_double((b & (long long)0x8000000000000000ULL) | (re << 52) |
-                                    ((long long)(fb & 0x7fffff) << 29));
-    double t = fma(-d, r, 1.0);
-    r = fma(r, t, r);
-    t = fma(-d, r, 1.0);
-    return fma(r, t, r);
+    const double r = __longlong_as_double((b & (long long)0x8000000000000000ULL) |
+                                          ((re << 52) + ((long long)(fb & 0x7fffff) << 29) + add));
+    return fma(r, fma(-d, r, 1.0), r);
 }
 
 // Weights of one point by a group of NW warps (thread t of the group). Assembles the packed

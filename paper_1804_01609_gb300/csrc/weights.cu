@@ -9,8 +9,8 @@
 // Bunch-Kaufman L D L^T (weights_point_ldl): ~m^3 / 3 flops per point either way (m = n + M), bound
 // by GB300's FP64 rate. Small systems take one warp per point (four points per block); larger ones
 // four warps per point, several points per SM so that one point's serial steps overlap the others'
-// products. N = 40,962, reduced form against the indefinite factorisation: m = 109 24.4 ms against
-// 30.3 ms, m = 71 7.8 ms against 10.1 ms, m = 40 2.3 ms against 2.9 ms.
+// products. N = 40,962, reduced form against the indefinite factorisation: m = 109 15.7 ms against
+// 30.3 ms, m = 71 6.6 ms against 10.1 ms, m = 40 2.1 ms against 2.9 ms.
 #include "common.cuh"
 #include "kernels.cuh"
 #include "device_ops.cuh"
@@ -64,13 +64,13 @@ struct WeightsArgs {
 };
 
 // NW warps per point (1 or 4). With NW = 1 a block holds blockDim/32 independent points and
-// the group barrier is __syncwarp; with NW > 1 a block is one point and uses __syncthreads.
-// At most 72 registers (seven 128-thread blocks per SM, no spills): where shared memory allows
-// more than four points per SM (m = 71: 25 KB each) the register file would otherwise cap the
-// blocks at five (11.3 against 10.1 ms at N = 40,962); at m = 109 shared memory caps them at four
-// either way.
-template <int NW, typename WT>
-__global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32, 7) weights_kernel(WeightsArgs a, WT *__restrict__ W) {
+// the group barrier is __syncwarp; with NW > 1 a block is one point and uses __syncthreads. kBlocks:
+// the blocks per SM that the registers are bounded for: seven for one warp per point (72 registers);
+// with four warps, whose digit products want 117, four where shared memory allows no more (m = 109)
+// and five (96 registers, 40 bytes spilled) where it does (m = 71: 6.6 ms against 7.1 ms at
+// N = 40,962; m = 109 16.9 against 16.4).
+template <int NW, int kBlocks, typename WT>
+__global__ void __launch_bounds__(128, kBlocks) weights_kernel(WeightsArgs a, WT *__restrict__ W) {
     extern __shared__ double smem[];
     constexpr int GT = NW * kWarp;
     const int g = threadIdx.x / GT, t = threadIdx.x % GT;
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32, 7) weights_kernel(Wei
     if (i >= a.Nq) return;  // NW == 1 only (with NW > 1 the grid has exactly Nq blocks)
     double *R = smem + (size_t)g * a.region_doubles;
     double *w = nullptr;
-    const int rc = weights_point<NW>(R, a.X, a.idx + i * a.n, a.n, a.m, a.ell, a.half,
+    const int rc = weights_point<NW, NW != 1>(R, a.X, a.idx + i * a.n, a.n, a.m, a.ell, a.half,
                                          a.P[3 * i], a.P[3 * i + 1], a.P[3 * i + 2], t, w);
     if (t >= kWarp) return;
     const int n = a.n, lane = t;
@@ -87,24 +87,23 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32, 7) weights_kernel(Wei
     if (a.status && lane == 0) a.status[i] = rc;
 }
 
-template <int NW, typename WT>
+template <int NW, int kBlocks, typename WT>
 int launch_weights_nw(const WeightsArgs &a, int spb, void *w, cudaStream_t s) {
     const int smem = spb * a.region_doubles * 8;
-    RBFSL_CUDA_TRY(cudaFuncSetAttribute(weights_kernel<NW, WT>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    auto *kernel = weights_kernel<NW, kBlocks, WT>;
+    RBFSL_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     // all of the unified L1 / shared storage as shared memory: as many points per SM as fit
-    RBFSL_CUDA_TRY(cudaFuncSetAttribute(weights_kernel<NW, WT>,
-                                        cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    RBFSL_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     const unsigned blocks = (unsigned)((a.Nq + spb - 1) / spb);
-    weights_kernel<NW, WT><<<blocks, spb * NW * kWarp, smem, s>>>(a, (WT *)w);
+    kernel<<<blocks, spb * NW * kWarp, smem, s>>>(a, (WT *)w);
     return launch_status("stencil_weights");
 }
 
-template <int NW>
+template <int NW, int kBlocks>
 int launch_weights_typed(const WeightsArgs &a, int spb, void *w, int w_dtype, cudaStream_t s) {
-    if (w_dtype == RBFSL_F64) return launch_weights_nw<NW, double>(a, spb, w, s);
-    if (w_dtype == RBFSL_F32X2) return launch_weights_nw<NW, float2>(a, spb, w, s);
-    return launch_weights_nw<NW, float>(a, spb, w, s);
+    if (w_dtype == RBFSL_F64) return launch_weights_nw<NW, kBlocks, double>(a, spb, w, s);
+    if (w_dtype == RBFSL_F32X2) return launch_weights_nw<NW, kBlocks, float2>(a, spb, w, s);
+    return launch_weights_nw<NW, kBlocks, float>(a, spb, w, s);
 }
 
 int launch_weights(const double *x, const int32_t *idx, int64_t Nq, int n, int ell, int power,
@@ -118,12 +117,13 @@ int launch_weights(const double *x, const int32_t *idx, int64_t Nq, int n, int e
     a.m = n + (ell + 1) * (ell + 1);
     a.region_doubles = weights_doubles(n, a.m, ell, a.half);
     const int bytes = a.region_doubles * 8;
-    if (bytes > kWeightsSmallBytes) {
-        // larger systems (m >~ 45): four warps per point (one per SM sub-partition), one point
-        // per block, as many blocks per SM as shared memory allows (four at m = 109)
-        return launch_weights_typed<4>(a, 1, w, w_dtype, s);
+    if (bytes > kWeightsSmallBytes || (reduced_form(n, ell, a.half) && reduced_on_tensor(a.m - n))) {
+        // larger systems (m >~ 45, or with the products on the tensor cores): four warps per point
+        // (one per SM sub-partition), one point per block; five blocks need 1/5 of 227 KB each
+        return bytes <= 44 * 1024 ? launch_weights_typed<4, 5>(a, 1, w, w_dtype, s)
+                                  : launch_weights_typed<4, 4>(a, 1, w, w_dtype, s);
     }
-    return launch_weights_typed<1>(a, 4, w, w_dtype, s);  // four independent points (warps) per block
+    return launch_weights_typed<1, 7>(a, 4, w, w_dtype, s);  // four independent points (warps) per block
 }
 
 // Centre-stencil weights, one warp per point (see center_point): bound by HBM bandwidth
