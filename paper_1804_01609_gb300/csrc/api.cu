@@ -84,6 +84,7 @@ struct rbfsl_ctx {
     double *xi = nullptr;
     int32_t *I = nullptr, *K = nullptr, *Ik = nullptr, *status = nullptr;
     void *W = nullptr;
+    CenterFactors center;               // centre stencils' factors
     unsigned long long *ctr = nullptr;  // [singular, knn failures]
     // prepared state (global method)
     double *LU = nullptr, *C64 = nullptr, *Q64 = nullptr;
@@ -149,6 +150,7 @@ void release_prepared(rbfsl_ctx *c) {
     c->knn = nullptr;
     cudaFree(c->xi); cudaFree(c->I); cudaFree(c->K); cudaFree(c->Ik); cudaFree(c->status);
     cudaFree(c->W); cudaFree(c->ctr);
+    center_factors_free(&c->center);
     c->xi = nullptr; c->I = c->K = c->Ik = c->status = nullptr; c->W = nullptr; c->ctr = nullptr;
     cudaFree(c->LU); cudaFree(c->C64); cudaFree(c->Q64); cudaFree(c->perm); cudaFree(c->piv);
     cudaFree(c->tc_ws); cudaFree(c->dev_err);
@@ -371,35 +373,12 @@ int prepare(rbfsl_ctx *c) {
     c->bytes += c->knn->bytes;
     if (c->mode == RBFSL_CENTER) {
         // stencil of node k: x_k and its n-1 nearest neighbours (Sec. 2.2), its saddle-point
-        // matrix factorised once (LU with partial pivoting, FP64; Sec. 3.3)
-        const int64_t m = n + (ell + 1) * (ell + 1);
+        // matrix factorised once (FP64; Sec. 3.3)
         if ((rc = dalloc(c, &c->K, N * sizeof(int32_t)))) return rc;
         if ((rc = dalloc(c, &c->Ik, N * n * sizeof(int32_t)))) return rc;
-        if ((rc = dalloc(c, &c->LU, N * m * m * sizeof(double)))) return rc;
-        if ((rc = dalloc(c, &c->perm, N * m * sizeof(int32_t)))) return rc;
         CTX_RC(c, launch_knn(c->knn, c->X, N, (int)n, c->Ik, c->status, c->stream));
-        std::vector<int64_t> ms(N + 1), lo(N);
-        for (int64_t k = 0; k <= N; ++k) ms[k] = k * n;
-        for (int64_t k = 0; k < N; ++k) lo[k] = k * m * m;
-        int64_t *d_ms = nullptr, *d_lo = nullptr;
-        int32_t *d_bad = nullptr;
-        CTX_TRY(c, cudaMalloc(&d_ms, (N + 1) * sizeof(int64_t)));
-        CTX_TRY(c, cudaMalloc(&d_lo, N * sizeof(int64_t)));
-        CTX_TRY(c, cudaMalloc(&d_bad, sizeof(int32_t)));
-        CTX_TRY(c, cudaMemcpy(d_ms, ms.data(), (N + 1) * sizeof(int64_t), cudaMemcpyHostToDevice));
-        CTX_TRY(c, cudaMemcpy(d_lo, lo.data(), N * sizeof(int64_t), cudaMemcpyHostToDevice));
-        CTX_TRY(c, cudaMemsetAsync(d_bad, 0, sizeof(int32_t), c->stream));
-        rc = launch_stencil_factor(c->X, d_ms, c->Ik, d_lo, N, (int)n, (ell + 1) * (ell + 1), ell, pw,
-                                   c->LU, c->perm, d_bad, c->stream, 1);
-        int32_t bad = 0;
-        if (rc == RBFSL_OK) {
-            cudaError_t e = cudaMemcpyAsync(&bad, d_bad, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-            if (e != cudaSuccess) rc = ctx_cuda(c, e, "centre factorisation");
-        }
-        cudaFree(d_ms); cudaFree(d_lo); cudaFree(d_bad);
-        if (rc != RBFSL_OK) return fail(c, rc, get_error());
-        if (bad) return fail(c, RBFSL_ESINGULAR, std::to_string(bad) + " singular centre stencils");
+        CTX_RC(c, center_factors_build(c->X, c->Ik, N, (int)n, ell, pw, &c->center, c->stream));
+        c->bytes += c->center.bytes;
     }
     c->prepared = true;
     return RBFSL_OK;
@@ -418,7 +397,7 @@ int one_step(rbfsl_ctx *c) {
         CTX_RC(c, launch_weights(c->X, c->I, N, n, ell, pw, c->xi, c->W, wdt, c->status, c->stream));
     } else {
         CTX_RC(c, launch_knn(c->knn, c->xi, N, 1, c->K, c->status, c->stream));
-        CTX_RC(c, launch_center_weights(c->X, c->K, c->Ik, c->LU, c->perm, N, n, ell, pw, c->xi, c->I, c->W,
+        CTX_RC(c, launch_center_weights(c->X, c->K, c->Ik, c->center, N, n, ell, pw, c->xi, c->I, c->W,
                                         wdt, c->status, c->stream));
     }
     count_status<<<(unsigned)((N + 255) / 256), 256, 0, c->stream>>>(c->status, N, c->ctr);

@@ -39,8 +39,9 @@ struct BatchDesc {
     int64_t step;
     const double *X;
     KnnGrid grid;
-    const double *LU;
-    const int32_t *perm, *Ik;
+    const double *F;         // centre stencils: factors and orders (CenterFactors)
+    const int32_t *order, *Ik;
+    int reduced;
     void *q[2];      // field ping-pong: input q[step & 1]
     double *xi;
     int32_t *status;
@@ -86,9 +87,11 @@ __global__ void batch_trace_kernel(const BatchDesc *__restrict__ d, int np, int6
 // int). Centre mode: right-hand side and solution (2 m double). The k-NN buffers (cap double +
 // cap int + 1 int) alias the start of the region: the search ends, and its result is copied
 // out, before the system or the right-hand side is written. A 109 x 109 system then takes
-// 55.6 KB, four points per SM.
+// 55.6 KB, four points per SM. (Centre mode with reduced factors: center_reduced_doubles.)
 __host__ __device__ inline int batch_region_doubles(int mode, int n, int m, int ell, int half) {
-    return mode == RBFSL_DIRECT ? weights_doubles(n, m, ell, half) + (n + 1) / 2 : 2 * m;
+    return mode == RBFSL_DIRECT ? weights_doubles(n, m, ell, half) + (n + 1) / 2
+         : reduced_form(n, ell, half) && center_reduced_doubles(n, m - n) > 2 * m ? center_reduced_doubles(n, m - n)
+                                                                                  : 2 * m;
 }
 __host__ __device__ inline int batch_point_doubles(int mode, int n, int m, int ell, int half, int cap) {
     const int region = batch_region_doubles(mode, n, m, ell, half), knn = cap + (cap + 2) / 2;
@@ -157,11 +160,16 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
                 if (rc == RBFSL_OK) batch_gather(b, wv, S, i, lane);
             } else {
                 const int64_t kc = bi[0];
+                __syncwarp();  // every lane has it before the region it lies in is overwritten
                 const int32_t *Sg = b.Ik + kc * n;
-                double *bb = A, *y = A + m;
-                center_point(b.X, Sg, b.LU + (size_t)kc * m * m, b.perm + (size_t)kc * m, n, m, b.ell, b.half,
-                             px, py, pz, bb, y, lane);
-                batch_gather(b, y, Sg, i, lane);
+                double *wv = A + m;
+                if (b.reduced)
+                    wv = center_point_reduced<32>(b.X, Sg, b.F + (size_t)kc * CenterLayout(n, m - n).total,
+                                                  b.order + (size_t)kc * n, n, m - n, b.ell, b.half, px, py, pz, A, lane);
+                else
+                    center_point(b.X, Sg, b.F + (size_t)kc * m * m, b.order + (size_t)kc * m, n, m, b.ell, b.half, px, py,
+                                 pz, A, wv, lane);
+                batch_gather(b, wv, Sg, i, lane);
             }
             if (rc != RBFSL_OK) {
                 const int in = (int)(b.step & 1);
@@ -238,8 +246,9 @@ struct HostProblem {
     bool used = false;
     BatchDesc d{};
     rbfsl_knn_index *knn = nullptr;
-    double *X = nullptr, *LU = nullptr, *xi = nullptr;
-    int32_t *perm = nullptr, *Ik = nullptr, *status = nullptr;
+    double *X = nullptr, *xi = nullptr;
+    int32_t *Ik = nullptr, *status = nullptr;
+    CenterFactors center;
     void *q[2] = {nullptr, nullptr};
     unsigned long long *ctr = nullptr;
     size_t bytes = 0;
@@ -285,7 +294,8 @@ int default_ppt(const rbfsl_batch *b, int n, int ell, int mode) {
 
 void free_problem(HostProblem &h) {
     if (h.knn) rbfsl_knn_index_destroy(h.knn);
-    cudaFree(h.X); cudaFree(h.LU); cudaFree(h.xi); cudaFree(h.perm); cudaFree(h.Ik);
+    center_factors_free(&h.center);
+    cudaFree(h.X); cudaFree(h.xi); cudaFree(h.Ik);
     cudaFree(h.status); cudaFree(h.q[0]); cudaFree(h.q[1]); cudaFree(h.ctr);
     h = HostProblem();
 }
@@ -524,40 +534,12 @@ int rbfsl_batch_add(rbfsl_batch *b, const rbfsl_problem *pr, int *id_out) {
     if ((rc = rbfsl_knn_index_create(&h.knn, h.X, N, pr->n, s))) { free_problem(h); return rc; }
     h.bytes += h.knn->bytes;
     if (pr->mode == RBFSL_CENTER) {
-        if ((rc = alloc((void **)&h.Ik, N * n * sizeof(int32_t))) ||
-            (rc = alloc((void **)&h.LU, (size_t)N * m * m * sizeof(double))) ||
-            (rc = alloc((void **)&h.perm, (size_t)N * m * sizeof(int32_t)))) {
+        if ((rc = alloc((void **)&h.Ik, N * n * sizeof(int32_t))) || (rc = launch_knn(h.knn, h.X, N, (int)n, h.Ik, h.status, s)) ||
+            (rc = center_factors_build(h.X, h.Ik, N, (int)n, pr->ell, pw, &h.center, s))) {
             free_problem(h);
             return rc;
         }
-        if ((rc = launch_knn(h.knn, h.X, N, (int)n, h.Ik, h.status, s))) { free_problem(h); return rc; }
-        std::vector<int64_t> ms(N + 1), lo(N);
-        for (int64_t k = 0; k <= N; ++k) ms[k] = k * n;
-        for (int64_t k = 0; k < N; ++k) lo[k] = k * (int64_t)m * m;
-        int64_t *d_ms = nullptr, *d_lo = nullptr;
-        int32_t *d_bad = nullptr;
-        if (cudaMalloc(&d_ms, (N + 1) * sizeof(int64_t)) != cudaSuccess || cudaMalloc(&d_lo, N * sizeof(int64_t)) != cudaSuccess ||
-            cudaMalloc(&d_bad, sizeof(int32_t)) != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(d_ms); cudaFree(d_lo);
-            free_problem(h);
-            set_error("batch_add: out of device memory");
-            return RBFSL_ENOMEM;
-        }
-        cudaMemcpyAsync(d_ms, ms.data(), (N + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_lo, lo.data(), N * sizeof(int64_t), cudaMemcpyHostToDevice, s);
-        cudaMemsetAsync(d_bad, 0, sizeof(int32_t), s);
-        rc = launch_stencil_factor(h.X, d_ms, h.Ik, d_lo, N, (int)n, M, pr->ell, pw, h.LU, h.perm, d_bad, s, 1);
-        int32_t bad = 0;
-        if (rc == RBFSL_OK && (cudaMemcpyAsync(&bad, d_bad, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-                               cudaStreamSynchronize(s) != cudaSuccess)) {
-            cudaGetLastError();
-            set_error("batch_add: centre factorisation failed");
-            rc = RBFSL_ECUDA;
-        }
-        cudaFree(d_ms); cudaFree(d_lo); cudaFree(d_bad);
-        if (rc == RBFSL_OK && bad) { set_error("batch_add: singular centre stencil"); rc = RBFSL_ESINGULAR; }
-        if (rc) { free_problem(h); return rc; }
+        h.bytes += h.center.bytes;
     }
     RBFSL_CUDA_TRY(cudaStreamSynchronize(s));
     BatchDesc &d = h.d;
@@ -566,7 +548,7 @@ int rbfsl_batch_add(rbfsl_batch *b, const rbfsl_problem *pr, int *id_out) {
     d.vel_kind = pr->vel_kind;
     for (int i = 0; i < 4; ++i) d.vel[i] = pr->vel_params[i];
     d.t = pr->t0; d.dt = pr->dt; d.step = 0;
-    d.X = h.X; d.grid = grid_view(h.knn); d.LU = h.LU; d.perm = h.perm; d.Ik = h.Ik;
+    d.X = h.X; d.grid = grid_view(h.knn); d.F = h.center.F; d.order = h.center.order; d.reduced = h.center.reduced; d.Ik = h.Ik;
     d.q[0] = h.q[0]; d.q[1] = h.q[1]; d.xi = h.xi; d.status = h.status; d.ctr = h.ctr;
     int id = -1;
     for (size_t i = 0; i < b->probs.size(); ++i)

@@ -97,10 +97,21 @@ int launch_stencil_factor(const double *X, const int64_t *mstart, const int32_t 
                           const int64_t *lu_off, int64_t count, int max_n, int M, int ell,
                           int power, double *LU, int32_t *perm, int32_t *status, cudaStream_t s,
                           int colmajor);
-int launch_center_weights(const double *X, const int32_t *K, const int32_t *Ik, const double *LU,
-                          const int32_t *perm, int64_t Nq, int n, int ell, int power,
-                          const double *p, int32_t *I, void *w, int w_dtype, int32_t *status,
-                          cudaStream_t s);
+
+// Kept factors of the centre stencils Ik (N x n): in the reduced form (reduced.cuh) or, where that
+// does not serve the system or breaks down at a stencil, LU of the whole systems.
+struct CenterFactors {
+    double *F = nullptr;       // per stencil: CenterLayout, or m x m column-major LU
+    int32_t *order = nullptr;  // per stencil: n (reduced) or m positions
+    int reduced = 0;
+    size_t bytes = 0;
+};
+int center_factors_build(const double *X, const int32_t *Ik, int64_t N, int n, int ell, int power,
+                         CenterFactors *out, cudaStream_t s);
+void center_factors_free(CenterFactors *f);
+int launch_center_weights(const double *X, const int32_t *K, const int32_t *Ik, const CenterFactors &f, int64_t Nq,
+                          int n, int ell, int power, const double *p, int32_t *I, void *w, int w_dtype,
+                          int32_t *status, cudaStream_t s);
 
 int global_factor_full(const double *x, int64_t N, int kernel, double eps, double *LU, int32_t *perm,
                        int32_t *piv, int32_t *status, cudaStream_t s);

@@ -64,6 +64,26 @@ struct RedLayout {
     }
 };
 
+// Stored factors of one centre stencil in the reduced form (doubles): the M x M factor of P1
+// (row-major: R above the diagonal, C below it, 1 / C_kk on it), then W, G = A21 - W A11 (K x M,
+// column-major), W^T (row k of W after the other) and B^-1 (K x K): n^2 + K M doubles, against the
+// (n + M)^2 of an LU factor of the whole system.
+struct CenterLayout {
+    int W, G, WT, Binv, total;
+    __host__ __device__ CenterLayout(int n, int M) {
+        const int K = n - M;
+        W = M * M;
+        G = W + K * M;
+        WT = G + K * M;
+        Binv = WT + K * M;
+        total = Binv + K * K;
+    }
+};
+__host__ __device__ inline int center_factor_doubles(int n, int ell, int half) {
+    const int M = (ell + 1) * (ell + 1);
+    return reduced_form(n, ell, half) ? CenterLayout(n, M).total : (n + M) * (n + M);
+}
+
 // Shared doubles of one point: the reduced form's region or the indefinite factorisation's (the
 // path of systems without the reduced form, and of a point whose reduced matrix breaks down),
 // whichever is larger.
@@ -95,6 +115,16 @@ __device__ __forceinline__ double sqrt_heron(double v) {
     return fma(fma(-g, g, v), hd, g);
 }
 
+// r^p = r (r^2)^half from r^2, the power by repeated squaring.
+__device__ __forceinline__ double phs_pow(double d2, int half) {
+    double v = sqrt_heron(d2), q = d2;
+    for (int h = half; h > 0; h >>= 1) {
+        if (h & 1) v *= q;
+        if (h > 1) q *= q;
+    }
+    return v;
+}
+
 __device__ __forceinline__ bool zero_or_not_finite(double v) {
     const long long b = __double_as_longlong(v) & 0x7fffffffffffffffLL;
     return b == 0 || b >= 0x7ff0000000000000LL;
@@ -105,11 +135,14 @@ __device__ __forceinline__ bool zero_or_not_finite(double v) {
 // NW gives the same bits. Returns RBFSL_OK with the weights (n doubles, stencil order) in `out`
 // (valid for warp 0), RBFSL_EKNN for a stencil index < 0, RBFSL_ESINGULAR for two coincident
 // stencil nodes, and 1 where a pivot of P or of B vanishes, is not finite or has the wrong sign.
-template <int NW, bool kTensor>
+// kFactor: instead of weights, store the factors that centre stencils keep (CenterLayout) at F and
+// the nodes' pivot order at order (p: any point, its row is not stored).
+template <int NW, bool kTensor, bool kFactor = false>
 __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, const double *__restrict__ X,
                                                      const int32_t *__restrict__ stencil, int n, int M, int ell,
                                                      int half, double px, double py, double pz, int t,
-                                                     double *&out) {
+                                                     double *&out, double *F = nullptr,
+                                                     int32_t *order = nullptr) {
     constexpr int GT = NW * kWarp;
     const int warp = t >> 5, lane = t & 31;
     const int n1 = n + 1, K = n - M, K1 = K + 1;
@@ -237,11 +270,7 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
         const double dx = cx[i] - cx[j], dy = cy[i] - cy[j], dz = cz[i] - cz[j];
         const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
         if (d2 == 0.0 && i < n) st[0] = RBFSL_ESINGULAR;  // two coincident nodes: two equal rows
-        double v = sqrt_heron(d2), q = d2;  // r^p = r (r^2)^half, the power by repeated squaring
-        for (int h = half; h > 0; h >>= 1) {
-            if (h & 1) v *= q;
-            if (h > 1) q *= q;
-        }
+        const double v = phs_pow(d2, half);
         if (i < M) {
             A11[tri(i - 1) + j] = v;
             if (kTensor) emax = max(emax, exp_field(v));
@@ -255,6 +284,30 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
     }
     gsync();
     if (st[0]) return st[0];
+    const CenterLayout fl(n, M);
+    if (kFactor) {  // P1's factor (reciprocal diagonal), W and its transpose, the order
+        for (int e = t; e < M * M; e += GT) {
+            const int k = e / M, j = e - k * M;
+            F[e] = j == k ? dinv[k] : P[j * S + k];
+        }
+        for (int e = t; e < M * K; e += GT) {
+            const int k = e / K, i = e - k * K;
+            const double w = P[k * S + M + i];
+            F[fl.W + e] = w;
+            F[fl.WT + i * M + k] = w;
+        }
+        for (int i = t; i < n; i += GT) order[i] = ord[i];
+        if (kTensor) gsync();
+    }
+    // A21 - W A11 = 2 Y - A21, with A21 formed again
+    auto store_g = [&] {
+        for (int e = t; e < M * K; e += GT) {
+            const int k = e / K, i = e - k * K, r = M + i;
+            const double dx = cx[r] - cx[k], dy = cy[r] - cy[k], dz = cz[r] - cz[k];
+            F[fl.G + e] = fma(2.0, Y[k * S2 + i], -phs_pow(fma(dz, dz, fma(dy, dy, dx * dx)), half));
+        }
+        gsync();
+    };
     const double *W = P + M;  // W[k * S + r]
     const int EW = kTensor ? st[2] + 1 : 0;
     if (kTensor) {
@@ -283,7 +336,7 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
             const double sc = split_scale(EW, EA);
             for (int tile = warp; tile < tm * ((M + 7) / 8); tile += NW) {
                 const int i0 = (tile % tm) * 16, j0 = (tile / tm) * 8, j = j0 + g;
-                float acc[kDigits][4] = {};
+                float acc[kGroups][4] = {};
                 for (int k0 = 0; k0 < M; k0 += 16)
                     split_mma(
                         acc, lane,
@@ -313,6 +366,7 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
         gsync();
         const int EY = st[4] + 1;
         if (EY >= 0x800 || !split_scale_ok(EW, EY)) return 1;
+        if (kFactor) store_g();
         to_digits(Y, S2, EY);
         gsync();
         const double sc = split_scale(EW, EY);
@@ -321,7 +375,7 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
             for (int ni = 0; ni < 2 * (mi + 1) && 8 * ni < K1; ++ni, ++tile) {
                 if (tile % NW != warp) continue;
                 const int i0 = 16 * mi, j = 8 * ni + g;
-                float acc[kDigits][4] = {};
+                float acc[kGroups][4] = {};
                 for (int k0 = 0; k0 < M; k0 += 16) {
                     auto wd = [&](int r, int k) { return r < K1 && k + k0 < M ? Wd[(k + k0) * S + r] : zero; };
                     auto yd = [&](int r, int k) { return r < K1 && k + k0 < M ? Yd[(k + k0) * S2 + r] : zero; };
@@ -347,6 +401,7 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
             Y[c * S2 + r] = fma(-0.5, acc, Y[c * S2 + r]);
         }
         gsync();
+        if (kFactor) store_g();
         // (lower triangle and the point's row; the point's own diagonal entry is unused)
         for (int e = t; e < tri(K1) - 1; e += GT) {
             const int i = tri_row(e), j = e - tri(i);
@@ -432,6 +487,24 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
         }
         gsync();
     }
+    if (kFactor) {
+        // ---- B^-1 = L^-T D^-1 L^-1, a thread per column, in place in global memory
+        for (int c = t; c < K; c += GT) {
+            double *x = F + fl.Binv + c;  // x_i at x[i * K]
+            for (int i = 0; i < K; ++i) {
+                const double *li = B + tri(i);
+                double a = i == c ? 1.0 : 0.0;
+                for (int j = c; j < i; ++j) a = fma(-li[j], x[j * K], a);
+                x[i * K] = i < c ? 0.0 : a;
+            }
+            for (int i = K - 1; i >= 0; --i) {
+                double a = i < c ? 0.0 : x[i * K] / B[tri(i) + i];
+                for (int j = i + 1; j < K; ++j) a = fma(-B[tri(j) + i], x[j * K], a);
+                x[i * K] = a;
+            }
+        }
+        return RBFSL_OK;
+    }
     if (warp != 0) return RBFSL_OK;
     // ---- L^T w2 = z (the last row of L), then w1 = u - W^T w2
     double *z = B + tri(K);
@@ -474,6 +547,95 @@ __device__ __forceinline__ int weights_point(double *__restrict__ R, const doubl
         if (NW == 1) __syncwarp(); else __syncthreads();  // every thread has read the breakdown flag
     }
     return weights_point_ldl<NW>(R, X, stencil, n, m, ell, half, px, py, pz, t, out);
+}
+
+// ---- Centre stencils (Sec. 3.3): the point uses the stencil of its nearest node, whose reduced
+// factors are kept. Per point u = P1^-T Y(p) by substitution with P1's factor, g = phi_2 - W phi_1 -
+// G u, w2 = B^-1 g and w1 = u - W^T w2: the last form keeps the weights' polynomial part exact
+// whatever the rounding of w2, so the inverse of B serves as well as its factors, and the three
+// products run without a serial chain. kLanes lanes of a warp per point.
+//
+// Bound: the FP64 pipe (two thirds of the multiplications of substituting through an LU factor of
+// the whole system, and a serial chain of 2 M steps instead of 2 (n + M)), then HBM (8 (n^2 + K M)
+// bytes per point). N = 40,962, n = 84 1.16 ms against 2.33 ms, N = 163,842, n = 31 0.91 ms against
+// 1.91 ms for the LU factors, which stay for the systems without the reduced form.
+
+// Shared doubles of one point: P1's factor, phi (later w2), Y(p), u, g and the weights.
+__host__ __device__ inline int center_reduced_doubles(int n, int M) { return M * M + 3 * n + M; }
+
+// Lanes per point: half a warp where the products then leave fewer lanes idle (K <= 32, M <= 16:
+// n = 31 has 22 and 9).
+__host__ __device__ inline int center_lanes(int n, int M) { return M <= 16 && n - M <= 32 ? 16 : 32; }
+
+// S: the stencil (n), F: its factors, order: pivot order; l: lane within the point's group. The
+// other groups of the warp run the same steps. Returns the weights (shared, stencil order).
+template <int kLanes>
+__device__ __forceinline__ double *center_point_reduced(const double *__restrict__ X, const int32_t *__restrict__ S,
+                                                        const double *__restrict__ F,
+                                                        const int32_t *__restrict__ order, int n, int M, int ell,
+                                                        int half, double px, double py, double pz,
+                                                        double *__restrict__ sm, int l) {
+    const int K = n - M;
+    const CenterLayout fl(n, M);
+    double *LU = sm, *phi = LU + M * M, *y = phi + n, *u = y + M, *g = u + M, *out = g + K;
+    for (int e = l; e < M * M; e += kLanes) LU[e] = F[e];
+    for (int j = l; j < n; j += kLanes) {
+        const int64_t s = S[order[j]];
+        const double dx = px - X[3 * s], dy = py - X[3 * s + 1], dz = pz - X[3 * s + 2];
+        phi[j] = phs_pow(fma(dz, dz, fma(dy, dy, dx * dx)), half);
+    }
+    sh_eval_lanes(ell, px, py, pz, l, [&](int c, double v) { y[c] = v; });
+    __syncwarp();
+    for (int k = 0; k < M; ++k) {  // y R^-1
+        const double yk = y[k];
+        for (int j = k + 1 + l; j < M; j += kLanes) y[j] = fma(-yk, LU[k * M + j], y[j]);
+        __syncwarp();
+    }
+    for (int k = M - 1; k >= 0; --k) {  // then C^-1
+        const double uk = y[k] * LU[k * M + k];
+        if (l == 0) u[k] = uk;
+        for (int j = l; j < k; j += kLanes) y[j] = fma(-uk, LU[k * M + j], y[j]);
+        __syncwarp();
+    }
+    for (int i = l; i < K; i += kLanes) {
+        const double *w = F + fl.W + i, *gg = F + fl.G + i;
+        double a0 = phi[M + i], a1 = 0.0;
+#pragma unroll 8
+        for (int k = 0; k < M; ++k) {
+            a0 = fma(-w[k * K], phi[k], a0);
+            a1 = fma(-gg[k * K], u[k], a1);
+        }
+        g[i] = a0 + a1;
+    }
+    __syncwarp();
+    for (int i = l; i < K; i += kLanes) {
+        const double *b = F + fl.Binv + i;
+        double a0 = 0.0, a1 = 0.0;
+        int j = 0;
+#pragma unroll 8
+        for (; j + 1 < K; j += 2) {
+            a0 = fma(b[j * K], g[j], a0);
+            a1 = fma(b[(j + 1) * K], g[j + 1], a1);
+        }
+        if (j < K) a0 = fma(b[j * K], g[j], a0);
+        phi[M + i] = a0 + a1;
+        out[order[M + i]] = a0 + a1;
+    }
+    __syncwarp();
+    for (int k = l; k < M; k += kLanes) {
+        const double *w = F + fl.WT + k, *z = phi + M;
+        double a0 = u[k], a1 = 0.0;
+        int i = 0;
+#pragma unroll 8
+        for (; i + 1 < K; i += 2) {
+            a0 = fma(-w[i * M], z[i], a0);
+            a1 = fma(-w[(i + 1) * M], z[i + 1], a1);
+        }
+        if (i < K) a0 = fma(-w[i * M], z[i], a0);
+        out[order[k]] = a0 + a1;
+    }
+    __syncwarp();
+    return out;
 }
 
 }  // namespace rbfsl

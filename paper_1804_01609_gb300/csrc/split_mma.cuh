@@ -3,15 +3,15 @@
 // exponent and cut into eight balanced base-256 digits, every digit exact in FP16. A product of
 // two digit matrices has integer entries, summed exactly by the FP32 accumulators while they stay
 // below 2^24; the digit products of equal weight (digit positions adding up to g) share one
-// accumulator. The 36 products of g <= 7 are kept: what is cut off is ~2^-57 of the largest entry
-// product, where an FP64 sum of 50 terms rounds at ~2^-52 of its partial sums.
+// accumulator. The 43 products of g <= 8 are kept: what is cut off is ~2^-65 of the largest entry
+// product (without g = 8, 2^-57: the weights of n = 84 stencils on 642 nodes then lost a digit).
 #pragma once
 
 #include "common.cuh"
 
 namespace rbfsl {
 
-constexpr int kDigits = 8;
+constexpr int kDigits = 8, kGroups = 9;
 
 // Field of x's exponent (biased, 0 for zero and subnormals, 0x7ff for infinities and NaN).
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
@@ -60,7 +60,7 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], c
 // acc[g] += the digit products of weight g of A (16 x 16) and B (16 x 8), one warp. A(r, k) for
 // r in {g, g + 8}, B(k): this lane's column; both return digits_of a number (0x8080...: zero).
 template <typename FA, typename FB>
-__device__ __forceinline__ void split_mma(float (&acc)[kDigits][4], int lane, FA A, FB B) {
+__device__ __forceinline__ void split_mma(float (&acc)[kGroups][4], int lane, FA A, FB B) {
     const int g = lane >> 2, t = (lane & 3) * 2;
     uint32_t b[kDigits][2];
     {
@@ -86,7 +86,7 @@ __device__ __forceinline__ void split_mma(float (&acc)[kDigits][4], int lane, FA
         const uint32_t a[4] = {digit_pair(x[0], x[1], s), digit_pair(x[4], x[5], s), digit_pair(x[2], x[3], s),
                                digit_pair(x[6], x[7], s)};
 #pragma unroll
-        for (int q = 0; q < kDigits - s; ++q) mma_f16(acc[s + q], a, b[q]);
+        for (int q = 0; q < kDigits && s + q < kGroups; ++q) mma_f16(acc[s + q], a, b[q]);
     }
 }
 
@@ -96,14 +96,15 @@ __device__ __forceinline__ double small_int_to_double(long long v) {
 }
 
 // The sum of the weighted accumulators of one entry, in units of 2^(EA + EB - 2 * 1023 - 34): the
-// exact integer hi 2^32 + lo rounded once (times 2^-32).
-__device__ __forceinline__ double split_value(const float (&acc)[kDigits][4], int u) {
+// exact integer hi 2^32 + lo rounded once (times 2^-32), the last group rounded into lo.
+__device__ __forceinline__ double split_value(const float (&acc)[kGroups][4], int u) {
     long long hi = 0, lo = 0;
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
         hi = hi * 256 + __float2int_rn(acc[g][u]);
         lo = lo * 256 + __float2int_rn(acc[g + 4][u]);
     }
+    lo += (__float2int_rn(acc[8][u]) + 128) >> 8;
     return fma(small_int_to_double(lo), 0x1p-32, small_int_to_double(hi));
 }
 

@@ -11,6 +11,8 @@
 // four warps per point, several points per SM so that one point's serial steps overlap the others'
 // products. N = 40,962, reduced form against the indefinite factorisation: m = 109 15.7 ms against
 // 30.3 ms, m = 71 6.6 ms against 10.1 ms, m = 40 2.1 ms against 2.9 ms.
+#include <vector>
+
 #include "common.cuh"
 #include "kernels.cuh"
 #include "device_ops.cuh"
@@ -126,8 +128,7 @@ int launch_weights(const double *x, const int32_t *idx, int64_t Nq, int n, int e
     return launch_weights_typed<1, 7>(a, 4, w, w_dtype, s);  // four independent points (warps) per block
 }
 
-// Centre-stencil weights, one warp per point (see center_point): bound by HBM bandwidth
-// (8 m^2 bytes of factor per point) and the FP64 rate (2 m^2 flops per point).
+// Centre-stencil weights from LU factors of the whole systems, one warp per point (center_point).
 template <typename WT>
 __global__ void __launch_bounds__(128) center_weights_kernel(
     const double *__restrict__ X, const int32_t *__restrict__ Kc, const int32_t *__restrict__ Ik,
@@ -153,25 +154,149 @@ __global__ void __launch_bounds__(128) center_weights_kernel(
     if (status && lane == 0) status[i] = RBFSL_OK;
 }
 
-int launch_center_weights(const double *X, const int32_t *K, const int32_t *Ik, const double *LU,
-                          const int32_t *perm, int64_t Nq, int n, int ell, int power,
-                          const double *p, int32_t *I, void *w, int w_dtype, int32_t *status,
-                          cudaStream_t s) {
+// The same from the reduced factors, kLanes lanes per point (center_point_reduced).
+template <typename WT, int kLanes>
+__global__ void __launch_bounds__(128) center_reduced_kernel(
+    const double *__restrict__ X, const int32_t *__restrict__ Kc, const int32_t *__restrict__ Ik,
+    const double *__restrict__ F, const int32_t *__restrict__ order, int64_t Nq, int n, int M, int ell, int half,
+    const double *__restrict__ P, int32_t *__restrict__ I, WT *__restrict__ W, int32_t *__restrict__ status) {
+    extern __shared__ double sm[];
+    const int grp = threadIdx.x / kLanes, l = threadIdx.x % kLanes;
+    const int64_t i0 = (int64_t)blockIdx.x * (128 / kLanes) + grp;
+    if (i0 - grp % (32 / kLanes) >= Nq) return;  // the whole warp past the end
+    const bool on = i0 < Nq;                     // a group past the end repeats the last point
+    const int64_t i = on ? i0 : Nq - 1;
+    const int64_t kc = Kc[i], k = kc < 0 ? 0 : kc;
+    const int32_t *S = Ik + k * n;
+    double *w = center_point_reduced<kLanes>(X, S, F + (size_t)k * CenterLayout(n, M).total, order + (size_t)k * n, n, M,
+                                             ell, half, P[3 * i], P[3 * i + 1], P[3 * i + 2],
+                                             sm + (size_t)grp * center_reduced_doubles(n, M), l);
+    if (!on) return;
+    for (int j = l; j < n; j += kLanes) {
+        W[i * n + j] = wcast<WT>(kc < 0 ? (double)NAN : w[j]);
+        I[i * n + j] = kc < 0 ? -1 : S[j];
+    }
+    if (status && l == 0) status[i] = kc < 0 ? RBFSL_EKNN : RBFSL_OK;
+}
+
+// Reduced factors of every stencil, one block per stencil. bad[0]: stencils without them, bad[1]:
+// failed neighbour searches.
+__global__ void __launch_bounds__(128, 4) center_factor_kernel(const double *__restrict__ X,
+                                                               const int32_t *__restrict__ Ik, int n, int M, int ell,
+                                                               int half, double *__restrict__ F,
+                                                               int32_t *__restrict__ order, int32_t *__restrict__ bad) {
+    extern __shared__ double sm[];
+    const int64_t k = blockIdx.x;
+    double *out = nullptr, *Fk = F + (size_t)k * CenterLayout(n, M).total;
+    const int32_t s0 = Ik[k * n];
+    const int64_t c = s0 < 0 ? 0 : s0;
+    const int t = threadIdx.x;
+    const int rc = reduced_on_tensor(M)
+                       ? weights_point_reduced<4, true, true>(sm, X, Ik + k * n, n, M, ell, half, X[3 * c], X[3 * c + 1],
+                                                              X[3 * c + 2], t, out, Fk, order + (size_t)k * n)
+                       : weights_point_reduced<4, false, true>(sm, X, Ik + k * n, n, M, ell, half, X[3 * c], X[3 * c + 1],
+                                                               X[3 * c + 2], t, out, Fk, order + (size_t)k * n);
+    if (t == 0 && rc != RBFSL_OK) atomicAdd(&bad[rc == RBFSL_EKNN ? 1 : 0], 1);
+}
+
+void center_factors_free(CenterFactors *f) {
+    cudaFree(f->F);
+    cudaFree(f->order);
+    *f = CenterFactors();
+}
+
+int center_factors_build(const double *X, const int32_t *Ik, int64_t N, int n, int ell, int power, CenterFactors *out,
+                         cudaStream_t s) {
+    int rc = sh_tables_init();
+    if (rc) return rc;
+    const int M = (ell + 1) * (ell + 1), m = n + M, half = (power - 1) / 2;
+    int32_t *bad = nullptr, hb[2] = {0, 0};
+    int64_t *csr = nullptr;
+    auto fail = [&](int code, const char *msg) {
+        cudaGetLastError();
+        cudaFree(bad);
+        cudaFree(csr);
+        center_factors_free(out);
+        set_error(msg);
+        return code;
+    };
+    auto read_bad = [&] {
+        return cudaMemcpyAsync(hb, bad, sizeof(hb), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
+               cudaStreamSynchronize(s) == cudaSuccess;
+    };
+    if (cudaMalloc(&bad, sizeof(hb)) != cudaSuccess) return fail(RBFSL_ENOMEM, "centre factors: out of device memory");
+    if (reduced_form(n, ell, half)) {
+        const size_t fb = (size_t)N * CenterLayout(n, M).total * sizeof(double), ob = (size_t)N * n * sizeof(int32_t);
+        if (cudaMalloc(&out->F, fb) != cudaSuccess || cudaMalloc(&out->order, ob) != cudaSuccess)
+            return fail(RBFSL_ENOMEM, "centre factors: out of device memory");
+        out->bytes = fb + ob;
+        out->reduced = 1;
+        const int smem = RedLayout(n, M).total * (int)sizeof(double);
+        if (cudaFuncSetAttribute(center_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+            cudaMemsetAsync(bad, 0, sizeof(hb), s) != cudaSuccess)
+            return fail(RBFSL_ECUDA, "centre factorisation failed");
+        center_factor_kernel<<<(unsigned)N, 128, smem, s>>>(X, Ik, n, M, ell, half, out->F, out->order, bad);
+        if (launch_status("center_factor") || !read_bad()) return fail(RBFSL_ECUDA, "centre factorisation failed");
+        if (hb[1]) return fail(RBFSL_EKNN, "centre stencils: the neighbour search failed");
+        if (!hb[0]) {
+            cudaFree(bad);
+            return RBFSL_OK;
+        }
+        center_factors_free(out);
+    }
+    // LU of the whole systems (partial pivoting, FP64)
+    const size_t fb = (size_t)N * m * m * sizeof(double), ob = (size_t)N * m * sizeof(int32_t);
+    if (cudaMalloc(&out->F, fb) != cudaSuccess || cudaMalloc(&out->order, ob) != cudaSuccess ||
+        cudaMalloc(&csr, (2 * N + 1) * sizeof(int64_t)) != cudaSuccess)
+        return fail(RBFSL_ENOMEM, "centre factors: out of device memory");
+    out->bytes = fb + ob;
+    out->reduced = 0;
+    std::vector<int64_t> h(2 * N + 1);
+    for (int64_t k = 0; k <= N; ++k) h[k] = k * n;
+    for (int64_t k = 0; k < N; ++k) h[N + 1 + k] = k * m * m;
+    if (cudaMemcpyAsync(csr, h.data(), h.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemsetAsync(bad, 0, sizeof(hb), s) != cudaSuccess)
+        return fail(RBFSL_ECUDA, "centre factorisation failed");
+    rc = launch_stencil_factor(X, csr, Ik, csr + N + 1, N, n, M, ell, power, out->F, out->order, bad, s, 1);
+    if (rc != RBFSL_OK || !read_bad()) return fail(rc ? rc : RBFSL_ECUDA, rc ? get_error() : "centre factorisation failed");
+    if (hb[0]) return fail(RBFSL_ESINGULAR, (std::to_string(hb[0]) + " singular centre stencils").c_str());
+    cudaFree(bad);
+    cudaFree(csr);
+    return RBFSL_OK;
+}
+
+namespace {
+template <typename WT>
+void launch_center_typed(const double *X, const int32_t *K, const int32_t *Ik, const CenterFactors &f, int64_t Nq, int n,
+                         int ell, int half, const double *p, int32_t *I, void *w, int32_t *status, cudaStream_t s) {
+    const int M = (ell + 1) * (ell + 1), m = n + M;
+    if (!f.reduced) {
+        center_weights_kernel<WT><<<(unsigned)((Nq + 3) / 4), 128, 4 * 2 * m * sizeof(double), s>>>(
+            X, K, Ik, f.F, f.order, Nq, n, ell, half, p, I, (WT *)w, status);
+        return;
+    }
+    const int lanes = center_lanes(n, M), ppb = 128 / lanes;
+    const int smem = ppb * center_reduced_doubles(n, M) * (int)sizeof(double);
+    auto go = [&](auto *kernel) {
+        if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        kernel<<<(unsigned)((Nq + ppb - 1) / ppb), 128, smem, s>>>(X, K, Ik, f.F, f.order, Nq, n, M, ell, half, p, I,
+                                                                  (WT *)w, status);
+    };
+    if (lanes == 16) go(center_reduced_kernel<WT, 16>);
+    else go(center_reduced_kernel<WT, 32>);
+}
+}  // namespace
+
+int launch_center_weights(const double *X, const int32_t *K, const int32_t *Ik, const CenterFactors &f, int64_t Nq,
+                          int n, int ell, int power, const double *p, int32_t *I, void *w, int w_dtype,
+                          int32_t *status, cudaStream_t s) {
     if (Nq == 0) return RBFSL_OK;
     int rc = sh_tables_init();
     if (rc) return rc;
-    const int m = n + (ell + 1) * (ell + 1);
-    const size_t smem = 4 * 2 * m * sizeof(double);
-    const unsigned blocks = (unsigned)((Nq + 3) / 4);
-    if (w_dtype == RBFSL_F64)
-        center_weights_kernel<double><<<blocks, 128, smem, s>>>(X, K, Ik, LU, perm, Nq, n, ell, (power - 1) / 2,
-                                                                p, I, (double *)w, status);
-    else if (w_dtype == RBFSL_F32X2)
-        center_weights_kernel<float2><<<blocks, 128, smem, s>>>(X, K, Ik, LU, perm, Nq, n, ell, (power - 1) / 2,
-                                                                p, I, (float2 *)w, status);
-    else
-        center_weights_kernel<float><<<blocks, 128, smem, s>>>(X, K, Ik, LU, perm, Nq, n, ell, (power - 1) / 2,
-                                                               p, I, (float *)w, status);
+    const int half = (power - 1) / 2;
+    if (w_dtype == RBFSL_F64) launch_center_typed<double>(X, K, Ik, f, Nq, n, ell, half, p, I, w, status, s);
+    else if (w_dtype == RBFSL_F32X2) launch_center_typed<float2>(X, K, Ik, f, Nq, n, ell, half, p, I, w, status, s);
+    else launch_center_typed<float>(X, K, Ik, f, Nq, n, ell, half, p, I, w, status, s);
     return launch_status("center_weights");
 }
 

@@ -9,6 +9,7 @@ torch = pytest.importorskip("torch")
 
 from paper_1804_01609_gb300 import inputs, rbfsl  # noqa: E402
 
+import _parity  # noqa: E402
 import test_gpu_local as loc  # noqa: E402
 
 pytestmark = pytest.mark.gpu
@@ -48,3 +49,34 @@ def test_rank_deficient_harmonics_are_singular():
     rbfsl.rbfsl_stencil_weights(loc._t(X), loc._t(I, torch.int32), n, 1, rbfsl.PHS, 3, loc._t(P), w, st)
     assert (st.cpu().numpy() == rbfsl.ESINGULAR).all()
     assert np.isnan(w.cpu().numpy()).all()
+
+
+# centre stencils: half a warp per point (K <= 32, M <= 16) with a ragged last block, a full warp,
+# products on both pipes, one node besides the pivots, and exponents that keep the LU factors
+@pytest.mark.parametrize("n,ell,p", [(31, 2, 5), (41, 2, 5), (42, 2, 5), (49, 3, 7), (84, 4, 9), (10, 2, 5), (17, 1, 3),
+                                     (31, 2, 9)])
+@pytest.mark.parametrize("prec", [rbfsl.FP64, rbfsl.MIXED])
+def test_centre_stencils_match_oracle(orc, n, ell, p, prec):
+    N, dt, steps = 901, 1.0 / 60, 3
+    X = inputs.nodes(N, 11)
+    vp = inputs.deformation_params(2.0, 1.0)
+    fields = inputs.TracerSet([lambda P: inputs.gaussian_hills(P, [[0.6, 0.0, 0.8], [0.0, 1.0, 0.0]]),
+                               lambda P: inputs.cosine_bell(P, [1.0, 0.0, 0.0], 0.9)])
+    q = fields(X)
+    c = rbfsl.Context(0)
+    c.set_nodes(X)
+    c.set_velocity(rbfsl.VEL_DEFORM_Y2, vp)
+    c.set_method(rbfsl.LOCAL, rbfsl.CENTER)
+    c.set_stencil_size(n)
+    c.set_sh_degree(ell)
+    c.set_kernel(rbfsl.PHS, p)
+    c.set_precision(prec)
+    c.set_dt(dt)
+    c.set_tracers(q)
+    c.step(steps)
+    got, st = c.get_q(), c.get_stats()
+    c.close()
+    assert st.singular_points == 0 and st.knn_failures == 0
+    ref = orc.local_run(X, q, n, ell, p, rbfsl.VEL_DEFORM_Y2, vp, dt, steps, mode=orc.CENTER)
+    exact = _parity.exact_field(fields, X, rbfsl.VEL_DEFORM_Y2, vp, steps * dt)
+    _parity.check_run(f"centre n={n} ell={ell} r^{p} prec={prec}", got, ref, exact, strict=False)
