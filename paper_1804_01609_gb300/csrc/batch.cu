@@ -85,7 +85,7 @@ __global__ void batch_trace_kernel(const BatchDesc *__restrict__ d, int np, int6
 
 // Shared memory of one point. Direct mode: system region (weights_doubles), then the stencil (n
 // int). Centre mode: right-hand side and solution (2 m double). The k-NN buffers (cap double +
-// cap int + 1 int) alias the start of the region: the search ends, and its result is copied
+// cap int) alias the start of the region: the search ends, and its result is copied
 // out, before the system or the right-hand side is written. A 109 x 109 system then takes
 // 55.6 KB, four points per SM. (Centre mode with reduced factors: center_reduced_doubles.)
 __host__ __device__ inline int batch_region_doubles(int mode, int n, int m, int ell, int half) {
@@ -94,7 +94,7 @@ __host__ __device__ inline int batch_region_doubles(int mode, int n, int m, int 
                                                                                   : 2 * m;
 }
 __host__ __device__ inline int batch_point_doubles(int mode, int n, int m, int ell, int half, int cap) {
-    const int region = batch_region_doubles(mode, n, m, ell, half), knn = cap + (cap + 2) / 2;
+    const int region = batch_region_doubles(mode, n, m, ell, half), knn = cap + (cap + 1) / 2;
     return region > knn ? region : knn;
 }
 
@@ -146,9 +146,8 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
             int32_t *S = reinterpret_cast<int32_t *>(base + weights_doubles(n, m, b.ell, b.half));  // direct only
             double *bd = base;  // aliases the region (see batch_point_doubles)
             int *bi = reinterpret_cast<int *>(bd + cap);
-            int *cnt = bi + cap;
             const double px = b.xi[3 * i], py = b.xi[3 * i + 1], pz = b.xi[3 * i + 2];
-            const bool ok = knn_warp(b.grid, px, py, pz, k, cap, bd, bi, cnt, lane);
+            const bool ok = knn_warp(b.grid, px, py, pz, k, cap, bd, bi, lane);
             int rc = RBFSL_OK;
             if (!ok) {
                 rc = RBFSL_EKNN;
@@ -186,10 +185,9 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
             int32_t *S = reinterpret_cast<int32_t *>(sm + weights_doubles(n, m, b.ell, b.half));
             double *bd = sm;  // aliases the region (see batch_point_doubles)
             int *bi = reinterpret_cast<int *>(bd + cap);
-            int *cnt = bi + cap;
             const double px = b.xi[3 * i], py = b.xi[3 * i + 1], pz = b.xi[3 * i + 2];
             if (warp == 0) {
-                const bool ok = knn_warp(b.grid, px, py, pz, k, cap, bd, bi, cnt, lane);
+                const bool ok = knn_warp(b.grid, px, py, pz, k, cap, bd, bi, lane);
                 for (int j = lane; j < n; j += 32) S[j] = ok ? bi[j] : -1;
             }
             __syncthreads();

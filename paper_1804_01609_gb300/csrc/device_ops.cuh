@@ -287,35 +287,47 @@ __device__ __forceinline__ bool key_less(long long da, int ia, long long db, int
 }
 
 // k nearest nodes of (qx, qy, qz) by one warp. bd/bi: the warp's candidate buffers (cap
-// entries, cap a power of two >= k), cnt: one shared int. On success bi[0..k) holds the node
-// indices ascending by (d2, index) and the function returns true; false if no radius in 40
-// rescalings brackets between k and cap candidates.
+// entries, cap a power of two >= k). On success bi[0..k) holds the node indices ascending by
+// (d2, index) and the function returns true; false if no radius in 40 rescalings brackets between
+// k and cap candidates. A single neighbour is kept in registers instead of a sorted list.
 __device__ __forceinline__ bool knn_warp(const KnnGrid &g, double qx, double qy, double qz, int k,
-                                         int cap, double *bd, int *bi, int *cnt, int lane) {
-    double r2 = g.r2_per_k * k;
+                                         int cap, double *bd, int *bi, int lane) {
+    // a ball that holds 1.3 k nodes on average; few neighbours take three more, so that the first
+    // ball is seldom empty
+    double r2 = g.r2_per_k * (k < 16 ? k + 3 : k);
     const double target = 1.3 * k;
-    long long r2b;  // r2 as key bits
+    const unsigned below = (1u << lane) - 1u;
     int total = 0;
     bool ok = false;
+    unsigned bh = 0xffffffffu, bl = 0xffffffffu;  // the nearest so far of this lane (k == 1)
+    int bn = 0x7fffffff;
     for (int iter = 0; iter < 40; ++iter) {
-        if (lane == 0) *cnt = 0;
-        __syncwarp();
+        total = 0;
         const double rb = sqrt(r2) * (1.0 + 1e-9) + 1e-15;
-        r2b = __double_as_longlong(r2);
-        grid_ball_foreach(g, qx, qy, qz, rb, lane, [&](int p) {
-            const double d2 = sqdist_rn(qx, qy, qz, g.sx[p], g.sy[p], g.sz[p]);
-            if (__double_as_longlong(d2) <= r2b) {  // d2 <= r2, both non-negative
-                const int slot = atomicAdd(cnt, 1);
-                if (slot < cap) {
-                    bd[slot] = d2;
-                    bi[slot] = g.sid[p];
+        const long long r2b = __double_as_longlong(r2);
+        grid_ball_foreach(g, qx, qy, qz, rb, lane, [&](int p, bool on) {
+            double d2 = 0.0;
+            if (on) {
+                d2 = sqdist_rn(qx, qy, qz, g.sx[p], g.sy[p], g.sz[p]);
+                on = __double_as_longlong(d2) <= r2b;  // d2 <= r2, both non-negative
+            }
+            const unsigned hit = __ballot_sync(0xffffffffu, on);
+            if (on) {
+                if (k == 1) {
+                    const unsigned h = (unsigned)__double2hiint(d2), l = (unsigned)__double2loint(d2);
+                    const int id = g.sid[p];
+                    if (h < bh || (h == bh && (l < bl || (l == bl && id < bn)))) { bh = h; bl = l; bn = id; }
+                } else {
+                    const int slot = total + __popc(hit & below);
+                    if (slot < cap) {
+                        bd[slot] = d2;
+                        bi[slot] = g.sid[p];
+                    }
                 }
             }
+            total += __popc(hit);
         });
-        __syncwarp();
-        total = *cnt;
-        __syncwarp();
-        if (total >= k && total <= cap) {
+        if (total >= k && (total <= cap || k == 1)) {
             ok = true;
             break;
         }
@@ -327,6 +339,14 @@ __device__ __forceinline__ bool knn_warp(const KnnGrid &g, double qx, double qy,
         r2 *= f;
     }
     if (!ok) return false;
+    if (k == 1) {
+        const unsigned mh = __reduce_min_sync(0xffffffffu, bh);
+        const unsigned ml = __reduce_min_sync(0xffffffffu, bh == mh ? bl : 0xffffffffu);
+        const unsigned mn = __reduce_min_sync(0xffffffffu, bh == mh && bl == ml ? (unsigned)bn : 0xffffffffu);
+        if (lane == 0) bi[0] = (int)mn;
+        __syncwarp();
+        return true;
+    }
     // Bitonic sort of the candidates by (d2, index), padded to a power of two.
     int P = 1;
     while (P < total) P <<= 1;
@@ -337,16 +357,14 @@ __device__ __forceinline__ bool knn_warp(const KnnGrid &g, double qx, double qy,
     __syncwarp();
     for (int len = 2; len <= P; len <<= 1) {
         for (int stride = len >> 1; stride > 0; stride >>= 1) {
-            for (int i = lane; i < P; i += kWarp) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    const bool up = (i & len) == 0;
-                    const double di = bd[i], dj = bd[j];
-                    const int ii = bi[i], ij = bi[j];
-                    if (key_less(__double_as_longlong(dj), ij, __double_as_longlong(di), ii) == up) {
-                        bd[i] = dj; bi[i] = ij;
-                        bd[j] = di; bi[j] = ii;
-                    }
+            for (int e = lane; e < P / 2; e += kWarp) {  // compare-exchange e: entries i and i + stride
+                const int i = ((e & ~(stride - 1)) << 1) | (e & (stride - 1)), j = i + stride;
+                const bool up = (i & len) == 0;
+                const double di = bd[i], dj = bd[j];
+                const int ii = bi[i], ij = bi[j];
+                if (key_less(__double_as_longlong(dj), ij, __double_as_longlong(di), ii) == up) {
+                    bd[i] = dj; bi[i] = ij;
+                    bd[j] = di; bi[j] = ii;
                 }
             }
             __syncwarp();

@@ -56,21 +56,61 @@ __device__ __forceinline__ int cell_coord(double v, double inv_cell, int G) {
     return c < 0 ? 0 : (c >= G ? G - 1 : c);
 }
 
-// Calls f(sorted_position) for every indexed point in the cells that overlap the ball of
-// radius rb around (qx, qy, qz); the cells are dealt to the lanes of a warp (lane, lane+32..).
+// Calls f(p, on) for the indexed points (sorted positions p, each once) of the cells that overlap the
+// ball of radius rb around (qx, qy, qz), 32 at a time: the whole warp calls f, on = false in lanes
+// without a point. The cells of a grid row (fixed y and z) are neighbours in the sorted order, so a
+// row's part of the ball is one range; the lanes take a row each, narrow its x-extent to the ball's
+// chord, and the ranges are dealt to the lanes point by point (a prefix sum of their lengths), so
+// that lanes idle in the last 32 only. A cell to a lane, with the whole bounding box, left most
+// lanes waiting for the few with occupied cells (k-NN, k = 84, N = 40,962: 984 us against 216 us).
+// Row and chord tests in FP32 with margins that cover its rounding: cells are only added. Cells on
+// the grid's border hold every point beyond it and are not narrowed on that side.
 template <typename F>
 __device__ __forceinline__ void grid_ball_foreach(const KnnGrid &g, double qx, double qy, double qz,
                                                   double rb, int lane, F f) {
-    const int x0 = cell_coord(qx - rb, g.inv_cell, g.G), x1 = cell_coord(qx + rb, g.inv_cell, g.G);
-    const int y0 = cell_coord(qy - rb, g.inv_cell, g.G), y1 = cell_coord(qy + rb, g.inv_cell, g.G);
-    const int z0 = cell_coord(qz - rb, g.inv_cell, g.G), z1 = cell_coord(qz + rb, g.inv_cell, g.G);
-    const int nx = x1 - x0 + 1, ny = y1 - y0 + 1, nz = z1 - z0 + 1;
-    const int nb = nx * ny * nz;
-    for (int t = lane; t < nb; t += 32) {
-        const int cx = x0 + t % nx, cy = y0 + (t / nx) % ny, cz = z0 + t / (nx * ny);
-        const int c = (cz * g.G + cy) * g.G + cx;
-        const int b = g.cell_start[c], e = g.cell_start[c + 1];
-        for (int p = b; p < e; ++p) f(p);
+    const float x = (float)qx, y = (float)qy, z = (float)qz, r = (float)rb * 1.00001f + 1e-6f;
+    const float inv = (float)g.inv_cell, edge = 1.0f / inv;
+    const int G = g.G;
+    auto cell = [&](float v, float margin) {
+        const int c = (int)floorf((v + 1.0f) * inv + margin);
+        return c < 0 ? 0 : (c >= G ? G - 1 : c);
+    };
+    auto outside = [&](float v, int c) {  // distance of v from cell c's interval
+        const float lo = c == 0 ? -1e30f : c * edge - 1.0f, hi = c == G - 1 ? 1e30f : (c + 1) * edge - 1.0f;
+        return fmaxf(fmaxf(lo - v, v - hi), 0.0f);
+    };
+    const int y0 = cell(y - r, -1e-3f), y1 = cell(y + r, 1e-3f), z0 = cell(z - r, -1e-3f), z1 = cell(z + r, 1e-3f);
+    const int ny = y1 - y0 + 1, rows = ny * (z1 - z0 + 1);
+    for (int base = 0; base < rows; base += 32) {
+        int b = 0, cnt = 0;
+        if (base + lane < rows) {
+            const int q = (base + lane) / ny, cz = z0 + q, cy = y0 + (base + lane - q * ny);
+            const float dy = outside(y, cy), dz = outside(z, cz);
+            const float h2 = r * r - dy * dy - dz * dz;
+            if (h2 >= -1e-4f * r * r) {
+                const float h = sqrtf(fmaxf(h2, 0.0f)) * 1.00001f + 0.02f * r;
+                const int64_t c = (int64_t)(cz * G + cy) * G;
+                b = g.cell_start[c + cell(x - h, -1e-3f)];
+                cnt = g.cell_start[c + cell(x + h, 1e-3f) + 1] - b;
+            }
+        }
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        for (int i0 = 0; i0 < total; i0 += 32) {
+            const int i = i0 + lane;
+            int row = 0;  // the first range that ends behind i
+#pragma unroll
+            for (int st = 16; st > 0; st >>= 1)
+                if (__shfl_sync(0xffffffffu, incl, row + st - 1) <= i) row += st;
+            row = row > 31 ? 31 : row;
+            const int p = __shfl_sync(0xffffffffu, b + cnt - incl, row) + i;
+            f(p, i < total);
+        }
     }
 }
 

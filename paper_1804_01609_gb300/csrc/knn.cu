@@ -127,7 +127,7 @@ void knn_index_free(rbfsl_knn_index *ix) {
     ix->sid = ix->cell_start = nullptr;
 }
 
-// One warp per query. Shared memory per warp: cap doubles + cap ints + 1 counter.
+// One warp per query. Shared memory per warp: cap doubles + cap ints.
 __global__ void __launch_bounds__(128) knn_query_kernel(KnnGrid g, const double *__restrict__ Q,
                                                         int64_t Nq, int k, int cap,
                                                         int32_t *__restrict__ idx,
@@ -138,11 +138,9 @@ __global__ void __launch_bounds__(128) knn_query_kernel(KnnGrid g, const double 
     double *bd = reinterpret_cast<double *>(smem_raw) + (size_t)warp * cap;
     int *bi = reinterpret_cast<int *>(reinterpret_cast<double *>(smem_raw) + (size_t)wpb * cap) +
               (size_t)warp * cap;
-    int *cnt = reinterpret_cast<int *>(reinterpret_cast<double *>(smem_raw) + (size_t)wpb * cap) +
-               (size_t)wpb * cap + warp;
     const int64_t q = (int64_t)blockIdx.x * wpb + warp;
     if (q >= Nq) return;
-    const bool ok = knn_warp(g, Q[3 * q], Q[3 * q + 1], Q[3 * q + 2], k, cap, bd, bi, cnt, lane);
+    const bool ok = knn_warp(g, Q[3 * q], Q[3 * q + 1], Q[3 * q + 2], k, cap, bd, bi, lane);
     for (int r = lane; r < k; r += kWarp) idx[q * k + r] = ok ? bi[r] : -1;
     if (status && lane == 0) status[q] = ok ? RBFSL_OK : RBFSL_EKNN;
 }
@@ -152,7 +150,7 @@ int launch_knn(const rbfsl_knn_index *ix, const double *q, int64_t Nq, int k, in
     if (Nq == 0) return RBFSL_OK;
     const int cap = knn_cap(k);
     const int wpb = 4;
-    const size_t smem = (size_t)wpb * cap * (sizeof(double) + sizeof(int)) + wpb * sizeof(int);
+    const size_t smem = (size_t)wpb * cap * (sizeof(double) + sizeof(int));
     const KnnGrid g = grid_view(ix);
     if (smem > 48 * 1024)
         RBFSL_CUDA_TRY(cudaFuncSetAttribute(knn_query_kernel,

@@ -47,9 +47,8 @@ __global__ void __launch_bounds__(128) pu_members_kernel(KnnGrid g, const double
     const double ox = Om[3 * l], oy = Om[3 * l + 1], oz = Om[3 * l + 2];
     if (lane == 0) cnt[warp] = 0;
     __syncwarp();
-    grid_ball_foreach(g, ox, oy, oz, R * (1.0 + 1e-9) + 1e-15, lane, [&](int p) {
-        const double d2 = sqdist_rn(ox, oy, oz, g.sx[p], g.sy[p], g.sz[p]);
-        if (sqrt(d2) < R) {
+    grid_ball_foreach(g, ox, oy, oz, R * (1.0 + 1e-9) + 1e-15, lane, [&](int p, bool on) {
+        if (on && sqrt(sqdist_rn(ox, oy, oz, g.sx[p], g.sy[p], g.sz[p])) < R) {
             const int slot = atomicAdd(&cnt[warp], 1);
             if (slot < kPuMaxCand) buf[warp][slot] = g.sid[p];
         }
@@ -240,8 +239,8 @@ __device__ __forceinline__ int pu_point_patches(const KnnGrid &cg, double Rr, in
                                                 double &wsum, int32_t *status, int64_t i, Fail fail) {
     if (lane == 0) sh.cnt[warp] = 0;
     __syncwarp();
-    grid_ball_foreach(cg, px, py, pz, Rr * (1.0 + 1e-9) + 1e-15, lane, [&](int p) {
-        const double d = sqrt(sqdist_rn(px, py, pz, cg.sx[p], cg.sy[p], cg.sz[p]));
+    grid_ball_foreach(cg, px, py, pz, Rr * (1.0 + 1e-9) + 1e-15, lane, [&](int p, bool on) {
+        const double d = on ? sqrt(sqdist_rn(px, py, pz, cg.sx[p], cg.sy[p], cg.sz[p])) : Rr;
         if (d < Rr) {
             const int slot = atomicAdd(&sh.cnt[warp], 1);
             if (slot < kPuMaxPatches) { sh.pl[warp][slot] = cg.sid[p]; sh.pd[warp][slot] = d; }
