@@ -8,6 +8,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "split_gemm.cuh"
 
 namespace rbfsl {
 
@@ -88,7 +89,8 @@ struct rbfsl_ctx {
     unsigned long long *ctr = nullptr;  // [singular, knn failures]
     // prepared state (global method)
     double *LU = nullptr, *C64 = nullptr, *Q64 = nullptr;
-    void *tc_ws = nullptr;     // global, mixed: tensor-core evaluation workspace
+    void *solve_factor = nullptr, *solve_ws = nullptr;  // the solve's inverted blocks and scratch
+    void *tc_ws = nullptr;     // global: evaluation workspace
     size_t tc_ws_bytes = 0;
     int32_t *dev_err = nullptr;  // RBFSL_ETIMEDOUT from a bounded device wait
     int32_t *perm = nullptr, *piv = nullptr;
@@ -153,6 +155,8 @@ void release_prepared(rbfsl_ctx *c) {
     center_factors_free(&c->center);
     c->xi = nullptr; c->I = c->K = c->Ik = c->status = nullptr; c->W = nullptr; c->ctr = nullptr;
     cudaFree(c->LU); cudaFree(c->C64); cudaFree(c->Q64); cudaFree(c->perm); cudaFree(c->piv);
+    cudaFree(c->solve_factor); cudaFree(c->solve_ws);
+    c->solve_factor = c->solve_ws = nullptr;
     cudaFree(c->tc_ws); cudaFree(c->dev_err);
     c->tc_ws = nullptr; c->tc_ws_bytes = 0; c->dev_err = nullptr;
     cudaFree(c->E); cudaFree(c->card_ws);
@@ -218,10 +222,15 @@ int prepare_global(rbfsl_ctx *c) {
     if (c->precision == RBFSL_MIXED) {
         if ((rc = dalloc(c, &c->Q64, N * T * sizeof(double)))) return rc;
         c->tc_ws_bytes = c->global_eval == RBFSL_GLOBAL_EVAL_TC ? global_eval_tc_workspace(N, N, (int)T)
-                                                                 : global_eval_pairs_workspace(N, N, (int)T);
-        if ((rc = dalloc(c, &c->tc_ws, c->tc_ws_bytes))) return rc;
+                                                                 : split_product_bytes(N, N, (int)T, RBFSL_F32X2);
+    } else {
+        c->tc_ws_bytes = split_product_bytes(N, N, (int)T, RBFSL_F64);
     }
+    if ((rc = dalloc(c, &c->tc_ws, c->tc_ws_bytes))) return rc;
+    if ((rc = dalloc(c, &c->solve_factor, split_solve_factor_bytes(N)))) return rc;
+    if ((rc = dalloc(c, &c->solve_ws, split_solve_scratch_bytes(N, (int)T)))) return rc;
     if ((rc = factor_global(c))) return rc;
+    CTX_RC(c, split_solve_prepare(c->LU, N, c->solve_factor, c->stream));
     c->prepared_T = c->T;
     c->prepared = true;
     return RBFSL_OK;
@@ -269,23 +278,26 @@ int one_step_global(rbfsl_ctx *c) {
     }
     const double t1 = c->t + c->dt;
     const unsigned blocks = (unsigned)((NT + 255) / 256);
+    auto solve = [&](const double *q) {
+        return split_solve(c->LU, c->perm, N, q, c->T, c->C64, c->solve_factor, c->solve_ws, c->stream);
+    };
     CTX_RC(c, launch_trace_order(c->X, N, c->vel_kind, c->vel, t1, c->dt, c->precision, c->integrator, c->xi, c->stream));
     if (c->precision == RBFSL_FP64) {
-        CTX_RC(c, global_solve(c->LU, c->perm, N, (const double *)c->q, c->T, c->C64, c->stream));
-        CTX_RC(c, launch_global_eval(c->xi, N, c->X, N, c->kkind, c->kparam, c->C64, c->T, RBFSL_F64,
-                                     c->q_next, RBFSL_F64, c->stream));
+        CTX_RC(c, solve((const double *)c->q));
+        CTX_RC(c, split_eval(c->xi, N, c->X, N, c->kkind, c->kparam, c->C64, c->T, RBFSL_F64, c->q_next, c->tc_ws,
+                             c->stream));
     } else if (c->global_eval == RBFSL_GLOBAL_EVAL_PAIRS) {
-        // FP64 solve of the field (FP32 pairs widened); kernel values in FP64, the sum in
-        // FP32-pair arithmetic, straight into the pair field
+        // FP64 solve of the field (FP32 pairs widened); kernel values in FP64, the sums rounded
+        // straight into the pair field
         from_pair_kernel<double><<<blocks, 256, 0, c->stream>>>((const float2 *)c->q, c->Q64, NT);
-        CTX_RC(c, global_solve(c->LU, c->perm, N, c->Q64, c->T, c->C64, c->stream));
-        CTX_RC(c, launch_global_eval_pairs(c->xi, N, c->X, N, c->kkind, c->kparam, c->C64, c->T,
-                                           (float2 *)c->q_next, c->tc_ws, c->tc_ws_bytes, c->stream));
+        CTX_RC(c, solve(c->Q64));
+        CTX_RC(c, split_eval(c->xi, N, c->X, N, c->kkind, c->kparam, c->C64, c->T, RBFSL_F32X2, c->q_next, c->tc_ws,
+                             c->stream));
     } else {
         // FP64 solve of the field (FP32 pairs widened); evaluation on the tensor cores (split
         // TF32, FP32 accumulation) into the freed FP64 right-hand side buffer, stored as pairs
         from_pair_kernel<double><<<blocks, 256, 0, c->stream>>>((const float2 *)c->q, c->Q64, NT);
-        CTX_RC(c, global_solve(c->LU, c->perm, N, c->Q64, c->T, c->C64, c->stream));
+        CTX_RC(c, solve(c->Q64));
         float *q32 = reinterpret_cast<float *>(c->Q64);
         CTX_RC(c, launch_global_eval_tc(c->xi, N, c->X, N, c->kkind, c->kparam, c->C64, RBFSL_F64, c->T, q32,
                                         c->tc_ws, c->dev_err, c->stream));

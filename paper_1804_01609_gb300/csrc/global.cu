@@ -16,14 +16,11 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "split_gemm.cuh"
 
 namespace rbfsl {
 
 constexpr int kNb = 64;  // panel / block size
-
-__device__ __forceinline__ double radial(int kind, double eps2, double d2) {
-    return kind == RBFSL_GAUSS ? exp(-eps2 * d2) : rsqrt(1.0 + eps2 * d2);
-}
 
 __global__ void global_assemble(const double *__restrict__ X, int64_t N, int kind, double eps2,
                                 double *__restrict__ A) {
@@ -31,7 +28,7 @@ __global__ void global_assemble(const double *__restrict__ X, int64_t N, int kin
     if (e >= N * N) return;
     const int64_t i = e / N, j = e - i * N;
     const double dx = X[3 * i] - X[3 * j], dy = X[3 * i + 1] - X[3 * j + 1], dz = X[3 * i + 2] - X[3 * j + 2];
-    A[e] = radial(kind, eps2, dx * dx + dy * dy + dz * dz);
+    A[e] = global_radial(kind, eps2, dx * dx + dy * dy + dz * dz);
 }
 
 // Pivot of column j (rows j..N-1), swap rows j and p inside the panel [j0, j0 + nb), scale the
@@ -429,8 +426,9 @@ __global__ void __launch_bounds__(kTrsmCols * 32) trsm_diag_col(const double *__
     if (lane + kWarp < nb) Y[(r0 + lane + kWarp) * T + c] = y1;
 }
 
-int global_solve(const double *LU, const int32_t *perm, int64_t N, const double *Q, int T,
-                 double *C, cudaStream_t s) {
+// Without scratch (see global_solve): blocks of 64, FP64 throughout.
+int global_solve_plain(const double *LU, const int32_t *perm, int64_t N, const double *Q, int T, double *C,
+                       cudaStream_t s) {
     const int64_t NT = N * T;
     gather_rows<<<(unsigned)((NT + 255) / 256), 256, 0, s>>>(Q, perm, N, T, C);
     // forward: L y = P q
@@ -450,6 +448,43 @@ int global_solve(const double *LU, const int32_t *perm, int64_t N, const double 
         if (rc) return rc;
     }
     return launch_status("global_solve");
+}
+
+namespace {
+
+// Stream-ordered scratch of one call; null where none can be had: under capture (a graph would keep
+// the allocation) or out of memory. The caller then takes the form without scratch.
+struct Scratch {
+    void *p = nullptr;
+    cudaStream_t s;
+    Scratch(size_t bytes, cudaStream_t st) : s(st) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+            cudaMallocAsync(&p, bytes, s) != cudaSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+    }
+    ~Scratch() {
+        if (p) cudaFreeAsync(p, s);
+    }
+    Scratch(const Scratch &) = delete;
+};
+
+}  // namespace
+
+// C = A_X^-1 Q, the solve's blocks inverted and its scratch taken for this call; systems of one
+// 64-row block have no trailing update to gain from.
+int global_solve(const double *LU, const int32_t *perm, int64_t N, const double *Q, int T, double *C, cudaStream_t s) {
+    if (N > kNb) {
+        const size_t fb = split_solve_factor_bytes(N);
+        Scratch ws(fb + split_solve_scratch_bytes(N, T), s);
+        if (ws.p) {
+            const int rc = split_solve_prepare(LU, N, ws.p, s);
+            return rc ? rc : split_solve(LU, perm, N, Q, T, C, ws.p, (char *)ws.p + fb, s);
+        }
+    }
+    return global_solve_plain(LU, perm, N, Q, T, C, s);
 }
 
 // ---- evaluation of the interpolant at Nq points: out[i][t] = sum_j phi(|p_i - x_j|) C[j][t]
@@ -484,7 +519,7 @@ __global__ void __launch_bounds__(TP * 8) global_eval_kernel(const double *__res
             if (j < N) {
                 if (sizeof(R) == 8) {
                     const double dx = ps[a][0] - X[3 * j], dy = ps[a][1] - X[3 * j + 1], dz = ps[a][2] - X[3 * j + 2];
-                    v = (R)radial(kind, eps2, dx * dx + dy * dy + dz * dz);
+                    v = (R)global_radial(kind, eps2, dx * dx + dy * dy + dz * dz);
                 } else {
                     const float dx = (float)ps[a][0] - (float)X[3 * j], dy = (float)ps[a][1] - (float)X[3 * j + 1],
                                 dz = (float)ps[a][2] - (float)X[3 * j + 2];
@@ -528,7 +563,9 @@ int launch_global_eval(const double *P, int64_t Nq, const double *X, int64_t N, 
     dim3 grid((unsigned)((Nq + 31) / 32), (unsigned)((T + 63) / 64));
     const double e2 = eps * eps;
     if (dtype == RBFSL_F64) {
-        // 8 points per block (64 threads): four times the blocks of 32, so that the FP64-bound
+        Scratch ws(split_product_bytes(Nq, N, T, RBFSL_F64), s);
+        if (ws.p) return split_eval(P, Nq, X, N, kind, eps, (const double *)C, T, RBFSL_F64, out, ws.p, s);
+        // without scratch, FP64 products: 8 points per block (64 threads): four times the blocks of 32, so that the FP64-bound
         // grid spreads evenly over the SMs (N = 10,242: 1,281 blocks instead of 321; 22.4 ->
         // 18.0 ms at T = 64)
         dim3 g8((unsigned)((Nq + 7) / 8), grid.y);
@@ -676,59 +713,11 @@ extern "C" int rbfsl_global_eval(const double *p, int64_t Nq, const double *x, i
 }
 
 // ---------------------------------------------------------------------------------------
-// FP64-accurate evaluation without FP64 products: the kernel matrix Phi(P, X) formed in FP64
-// (the same radial function and distance operations as the FP64 evaluation) and stored as FP32
-// pairs, the coefficients split into pairs, then Phi C by the FP32-pair product of the cardinal
-// form (rbfsl_cardinal_apply): ~2^-48 relative per term against the split-TF32 evaluation's
-// ~2^-22, at a fraction of the FP64 products' cost.
-namespace rbfsl {
-
-__global__ void phi_pairs_kernel(const double *__restrict__ P, int64_t Nq, const double *__restrict__ X, int64_t N,
-                                 int kind, double eps2, float2 *__restrict__ E) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= Nq * N) return;
-    const int64_t i = e / N, j = e - i * N;
-    const double dx = P[3 * i] - X[3 * j], dy = P[3 * i + 1] - X[3 * j + 1], dz = P[3 * i + 2] - X[3 * j + 2];
-    E[e] = pair_from(radial(kind, eps2, dx * dx + dy * dy + dz * dz));
-}
-
-__global__ void f64_to_pairs(const double *__restrict__ in, float2 *__restrict__ out, int64_t n) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e < n) out[e] = pair_from(in[e]);
-}
-
-size_t global_eval_pairs_workspace(int64_t Nq, int64_t N, int T) {
-    const size_t phi = ((size_t)Nq * N * sizeof(float2) + 255) & ~(size_t)255;
-    const size_t cp = ((size_t)N * T * sizeof(float2) + 255) & ~(size_t)255;
-    return phi + cp + cardinal_apply_workspace(Nq, N, T);
-}
-
-int launch_global_eval_pairs(const double *P, int64_t Nq, const double *X, int64_t N, int kind, double eps,
-                             const double *C, int T, float2 *out, void *ws, size_t ws_bytes, cudaStream_t s) {
-    if (Nq == 0) return RBFSL_OK;
-    const size_t need = global_eval_pairs_workspace(Nq, N, T);
-    if (!ws || ws_bytes < need) {
-        set_error("global_eval_pairs: workspace too small");
-        return RBFSL_EINVAL;
-    }
-    float2 *E = (float2 *)ws;
-    const size_t phi = ((size_t)Nq * N * sizeof(float2) + 255) & ~(size_t)255;
-    float2 *Cp = (float2 *)((char *)ws + phi);
-    const size_t cp = ((size_t)N * T * sizeof(float2) + 255) & ~(size_t)255;
-    void *aws = (char *)ws + phi + cp;
-    const int64_t ne = Nq * N, nc = N * (int64_t)T;
-    phi_pairs_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(P, Nq, X, N, kind, eps * eps, E);
-    f64_to_pairs<<<(unsigned)((nc + 255) / 256), 256, 0, s>>>(C, Cp, nc);
-    int rc = launch_status("global_eval_pairs");
-    if (rc) return rc;
-    return launch_cardinal_apply(E, Nq, N, Cp, T, RBFSL_F32X2, out, aws, ws_bytes - phi - cp, s);
-}
-
-}  // namespace rbfsl
-
+// FP64-accurate evaluation stored as FP32 pairs: kernel values formed in FP64, the products on the
+// tensor cores (split_gemm.cu), the sums rounded to pairs.
 extern "C" size_t rbfsl_global_eval_pairs_workspace_bytes(int64_t Nq, int64_t N, int T) {
     if (Nq < 0 || N < 1 || T < 1) return 0;
-    return rbfsl::global_eval_pairs_workspace(Nq, N, T);
+    return rbfsl::split_product_bytes(Nq, N, T, RBFSL_F32X2);
 }
 
 extern "C" int rbfsl_global_eval_pairs(const double *p, int64_t Nq, const double *x, int64_t N, int kernel,
@@ -739,8 +728,9 @@ extern "C" int rbfsl_global_eval_pairs(const double *p, int64_t Nq, const double
     RBFSL_CHECK_ARG(Nq == 0 || (p && x && c && out && workspace), "global_eval_pairs: null pointer");
     RBFSL_CHECK_ARG((kernel == RBFSL_GAUSS || kernel == RBFSL_IMQ) && eps > 0, "global_eval_pairs: bad kernel");
     RBFSL_CHECK_ARG(((uintptr_t)workspace & 255) == 0, "global_eval_pairs: workspace must be 256-byte aligned");
-    return launch_global_eval_pairs(p, Nq, x, N, kernel, eps, c, T, (float2 *)out, workspace, workspace_bytes,
-                                    (cudaStream_t)stream);
+    if (Nq == 0) return RBFSL_OK;
+    RBFSL_CHECK_ARG(workspace_bytes >= split_product_bytes(Nq, N, T, RBFSL_F32X2), "global_eval_pairs: workspace too small");
+    return split_eval(p, Nq, x, N, kernel, eps, c, T, RBFSL_F32X2, out, workspace, (cudaStream_t)stream);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -1,0 +1,506 @@
+// Dense products out = A x to FP64 accuracy on the tensor cores (split_mma.cuh), for the three
+// places of the global method that an FP64 product bounds: the trailing updates of the triangular
+// solves (A: strips of the factor), the evaluation (A: kernel values formed on the way) and the
+// cardinal form (A: the stored cardinal matrix, FP64 or FP32 pairs).
+//
+// The inner dimension is walked in chunks of 128: up to there the digit sums stay exact in the FP32
+// accumulators (128 terms x 8 products x 2^14 = 2^24). Each chunk's sums are scaled by the row's and
+// the column's own largest exponent of the chunk and added in FP64. x is cut into digits once
+// (x_digits); A's rows are cut by the block that uses them: a warp reads a row's 128 entries, takes
+// their largest exponent with one redux and leaves the digits in shared memory.
+//
+// Blocks of four warps: 16 rows x 32 columns per warp, as 2 x 2 warps (32 rows x 64 columns) or,
+// for up to 32 columns, 4 x 1 (64 rows). Bound: the tensor cores' FP16 rate, 43 digit products per
+// useful one (43 N^2 T / 304 TMAC/s: 0.95 ms at N = 10,242, T = 64, where the FP64 pipe takes
+// 10.7 ms), for few columns the digit extraction and the A stream.
+#include <algorithm>
+#include <type_traits>
+
+#include "common.cuh"
+#include "kernels.cuh"
+#include "split_gemm.cuh"
+#include "split_mma.cuh"
+
+namespace rbfsl {
+
+namespace {
+
+constexpr int kChunk = kSplitChunk;
+constexpr int kLd = 136;  // shared row of a chunk's digits (16-byte loads of eight rows hit all banks)
+constexpr int kEMin = 64, kENan = 0x7ff;
+
+// ---- sources of A: raw 64-bit words, their exponent field, their digits, their value
+struct SrcF64 {
+    const double *A;
+    int64_t ld;
+    __device__ __forceinline__ unsigned long long raw(int64_t r, int64_t k) const {
+        return (unsigned long long)__double_as_longlong(A[r * ld + k]);
+    }
+    __device__ __forceinline__ static int field(unsigned long long w) { return (int)(w >> 52) & 0x7ff; }
+    __device__ __forceinline__ static unsigned long long digits(unsigned long long w, int E) {
+        return digits_of(__longlong_as_double((long long)w), E);
+    }
+    __device__ __forceinline__ static double value(unsigned long long w) { return __longlong_as_double((long long)w); }
+};
+
+// v (a float) as a multiple of 2^(E - 1023 - 61), truncated (no byte bias).
+__device__ __forceinline__ long long fixed_of(uint32_t w, int E) {
+    const int e = (int)(w >> 23) & 0xff;
+    const long long m = (w & 0x7fffff) | (e ? 1u << 23 : 0u);
+    // m 2^(e' - 150) with e' = max(e, 1): shift 61 + 1023 - 150 - E + e'
+    const int s = (e ? e : 1) + 934 - E;
+    const long long v = s >= 0 ? m << (s > 40 ? 40 : s) : (s > -63 ? m >> -s : 0);
+    return (int)w < 0 ? -v : v;
+}
+
+struct SrcPair {
+    const float2 *A;
+    int64_t ld;
+    __device__ __forceinline__ unsigned long long raw(int64_t r, int64_t k) const {
+        const float2 v = A[r * ld + k];
+        return (unsigned long long)__float_as_uint(v.x) | (unsigned long long)__float_as_uint(v.y) << 32;
+    }
+    __device__ __forceinline__ static int field(unsigned long long w) {  // of the high part; not finite in either: kENan
+        const int e = (int)(w >> 23) & 0xff, f = (int)(w >> 55) & 0xff;
+        return e == 0xff || f == 0xff ? kENan : (e > f ? e : f) + 896;  // (a normalised pair has e >= f)
+    }
+    __device__ __forceinline__ static unsigned long long digits(unsigned long long w, int E) {
+        return (unsigned long long)(fixed_of((uint32_t)w, E) + fixed_of((uint32_t)(w >> 32), E)) + 0x8080808080808080ULL;
+    }
+    __device__ __forceinline__ static double value(unsigned long long w) {
+        return (double)__uint_as_float((uint32_t)w) + (double)__uint_as_float((uint32_t)(w >> 32));
+    }
+};
+
+struct SrcPhi : SrcF64 {
+    const double *P, *X;
+    int kind;
+    double eps2;
+    __device__ __forceinline__ unsigned long long raw(int64_t r, int64_t k) const {
+        const double dx = P[3 * r] - X[3 * k], dy = P[3 * r + 1] - X[3 * k + 1], dz = P[3 * r + 2] - X[3 * k + 2];
+        return (unsigned long long)__double_as_longlong(
+            global_radial(kind, eps2, fma(dz, dz, fma(dy, dy, dx * dx))));
+    }
+};
+
+__device__ __forceinline__ double x_value(const double *x) { return *x; }
+__device__ __forceinline__ double x_value(const float2 *x) { return (double)x->x + (double)x->y; }
+
+// Digits of x (K x T, row-major), chunk blockIdx.x, columns blockIdx.y * 32 .. + 32: D[chunk][k][t]
+// (row length Tp), the columns' exponents Ex[chunk][t] (largest field + 1, at least kEMin; not finite:
+// above kENan) and their largest, Ex[chunk][Tp] (zeroed by the caller).
+template <typename V>
+__global__ void __launch_bounds__(256) x_digits(const V *__restrict__ x, int64_t K, int T, int Tp,
+                                                unsigned long long *__restrict__ D, int *__restrict__ Ex) {
+    __shared__ int emax[32];
+    const int c = threadIdx.x & 31, w = threadIdx.x >> 5, t = blockIdx.y * 32 + c;
+    const int64_t ch = blockIdx.x, k0 = ch * kChunk;
+    if (threadIdx.x < 32) emax[threadIdx.x] = 0;
+    __syncthreads();
+    double v[kChunk / 8];
+    int e = 0;
+#pragma unroll
+    for (int u = 0; u < kChunk / 8; ++u) {
+        const int64_t k = k0 + w + 8 * u;
+        v[u] = k < K && t < T ? x_value(x + k * T + t) : 0.0;
+        e = max(e, exp_field(v[u]));
+    }
+    atomicMax(&emax[c], e);
+    __syncthreads();
+    const int E = max(emax[c] + 1, kEMin);
+    if (t < Tp) {
+#pragma unroll
+        for (int u = 0; u < kChunk / 8; ++u) D[(k0 + w + 8 * u) * Tp + t] = digits_of(v[u], E);
+        if (w == 0) {
+            Ex[ch * (Tp + 1) + t] = E;
+            atomicMax(&Ex[ch * (Tp + 1) + Tp], E);
+        }
+    }
+}
+
+// Scale of a chunk's sums: 2^(EA + EX - 2 * 1023 - 34), 0 where it is below the normal doubles.
+__device__ __forceinline__ double chunk_scale(int EA, int EX) {
+    const int e = EA + EX - 1023 - 34;
+    return __longlong_as_double((long long)(e > 0 ? e : 0) << 52);
+}
+
+// kSub: C[r][t] -= sum; else to out (row length T) + split * M * T.
+template <typename Src, typename V, int kWarpRows, bool kSub>
+__global__ void __launch_bounds__(128, 3) split_gemm_kernel(Src A, int64_t M, int64_t K, const V *__restrict__ x, int T,
+                                                            int Tp, const unsigned long long *__restrict__ D,
+                                                            const int *__restrict__ Ex, int nchunk, int span,
+                                                            double *__restrict__ out) {
+    constexpr int kRows = 16 * kWarpRows, kWarpCols = 4 / kWarpRows;
+    extern __shared__ __align__(16) unsigned long long As[];  // kRows x kLd digits
+    __shared__ int Er[kRows];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t2 = (lane & 3) * 2;
+    const int64_t r0 = (int64_t)blockIdx.x * kRows;
+    const int wr = (warp / kWarpCols) * 16, col0 = (blockIdx.y * kWarpCols + warp % kWarpCols) * 32;
+    const int c0 = blockIdx.z * span, c1 = min(nchunk, c0 + span);
+    double sum[4][4] = {};
+    for (int ch = c0; ch < c1; ++ch) {
+        const int64_t k0 = (int64_t)ch * kChunk;
+        const int kc = (int)min((int64_t)kChunk, K - k0);
+        // ---- digits of the block's rows, four rows of a warp at a time
+        bool bad = false;
+        const int exm = Ex[(int64_t)ch * (Tp + 1) + Tp];
+        for (int q = 0; q < kRows / 4; q += 4) {
+            unsigned long long w[4][4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int64_t r = r0 + warp * (kRows / 4) + q + v;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int k = lane + 32 * u;
+                    w[v][u] = r < M && k < kc ? A.raw(r, k0 + k) : 0ULL;
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int row = warp * (kRows / 4) + q + v;
+                int e = 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) e = max(e, Src::field(w[v][u]));
+                e = __reduce_max_sync(0xffffffffu, e);
+                const int E = max(e + 1, kEMin);
+                if (lane == 0) Er[row] = E;
+                bad |= e >= kENan || exm > kENan || E + exm >= 2047 + 1023 + 34;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) As[row * kLd + lane + 32 * u] = Src::digits(w[v][u], E);
+            }
+        }
+        if (__syncthreads_or(bad)) {
+            // not finite, or beyond the doubles' range: this chunk in plain FP64
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int64_t r = r0 + wr + g + 8 * (u >> 1);
+                    const int t = col0 + 8 * nt + t2 + (u & 1);
+                    if (r < M && t < T)
+#pragma unroll 1
+                        for (int k = 0; k < kc; ++k)
+                            sum[nt][u] = fma(Src::value(A.raw(r, k0 + k)), x_value(x + (k0 + k) * T + t), sum[nt][u]);
+                }
+        } else {
+#pragma unroll
+            for (int np = 0; np < 2; ++np) {  // two 8-column tiles at a time
+                const int cb = col0 + 16 * np;
+                if (cb >= Tp) break;
+                const bool two = cb + 8 < Tp;
+                float acc[2][kGroups][4] = {};
+                for (int ks = 0; ks * 16 < kc; ++ks) {
+                    const unsigned long long *a = As + (wr + g) * kLd + ks * 16 + t2;
+                    const ulonglong2 a0 = *reinterpret_cast<const ulonglong2 *>(a),
+                                     a1 = *reinterpret_cast<const ulonglong2 *>(a + 8 * kLd),
+                                     a2 = *reinterpret_cast<const ulonglong2 *>(a + 8),
+                                     a3 = *reinterpret_cast<const ulonglong2 *>(a + 8 * kLd + 8);
+                    const unsigned long long *d = D + (k0 + ks * 16 + t2) * Tp + cb + g;
+                    uint32_t b[2][kDigits][2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (h == 1 && !two) break;
+                        const unsigned long long b0 = d[8 * h], b1 = d[Tp + 8 * h], b2 = d[8 * Tp + 8 * h],
+                                                 b3 = d[9 * Tp + 8 * h];
+#pragma unroll
+                        for (int s = 0; s < kDigits; ++s) {
+                            b[h][s][0] = digit_pair(b0, b1, s);
+                            b[h][s][1] = digit_pair(b2, b3, s);
+                        }
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int s = 0; s < kDigits; ++s) {
+                        const uint32_t af[4] = {digit_pair(a0.x, a0.y, s), digit_pair(a1.x, a1.y, s),
+                                                digit_pair(a2.x, a2.y, s), digit_pair(a3.x, a3.y, s)};
+#pragma unroll
+                        for (int q = 0; q < kDigits && s + q < kGroups; ++q) {
+                            mma_f16(acc[0][s + q], af, b[0][q]);
+                            if (two) mma_f16(acc[1][s + q], af, b[1][q]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (h == 1 && !two) break;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int ea = Er[wr + g + 8 * (u >> 1)],
+                                  ex = Ex[(int64_t)ch * (Tp + 1) + cb + 8 * h + t2 + (u & 1)];
+                        sum[2 * np + h][u] = fma(split_value(acc[h], u), chunk_scale(ea, ex), sum[2 * np + h][u]);
+                    }
+                }
+            }
+        }
+        __syncthreads();  // the digits are read; the next chunk overwrites them
+    }
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t r = r0 + wr + g + 8 * (u >> 1);
+            const int t = col0 + 8 * nt + t2 + (u & 1);
+            if (r >= M || t >= T) continue;
+            if (kSub) out[r * T + t] -= sum[nt][u];
+            else out[((int64_t)blockIdx.z * M + r) * T + t] = sum[nt][u];
+        }
+}
+
+template <typename Src, typename V, bool kSub>
+int launch_gemm(const Src &A, int64_t M, int64_t K, const V *x, int T, int Tp, const unsigned long long *D, const int *Ex,
+                int splits, double *out, cudaStream_t s) {
+    const int nchunk = (int)((K + kChunk - 1) / kChunk), span = (nchunk + splits - 1) / splits;
+    auto go = [&](auto *kernel, int rows, int cols) {
+        const int smem = rows * kLd * 8;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return;
+        dim3 grid((unsigned)((M + rows - 1) / rows), (unsigned)((T + cols - 1) / cols), (unsigned)splits);
+        kernel<<<grid, 128, smem, s>>>(A, M, K, x, T, Tp, D, Ex, nchunk, span, out);
+    };
+    if (T <= 32) go(split_gemm_kernel<Src, V, 4, kSub>, 64, 32);
+    else go(split_gemm_kernel<Src, V, 2, kSub>, 32, 64);
+    return launch_status("split_gemm");
+}
+
+// ---- triangular solves with diagonal blocks of 128 rows
+constexpr int kB = 64;  // inverted triangular blocks (two to a diagonal block)
+
+// Inverses of the 64 x 64 diagonal blocks of the unit lower (blockIdx.y = 0) and the upper factor
+// (1), column-major, and the 64 x 64 block that couples a diagonal block's halves (also
+// column-major): what the block substitution needs, laid out for its lanes. A block's inverse
+// replaces 64 dependent steps by a product. Rows and columns beyond N: the identity.
+__global__ void __launch_bounds__(64) solve_prepare(const double *__restrict__ LU, int64_t N, double *__restrict__ inv,
+                                                    double *__restrict__ off) {
+    extern __shared__ double sm[];
+    double *F = sm, *V = sm + kB * (kB + 1);  // the block (row-major) and its inverse (column-major), padded
+    const int64_t j = blockIdx.x, r0 = j * kB;
+    const int c = threadIdx.x, upper = blockIdx.y;
+    for (int i = 0; i < kB; ++i)
+        F[i * (kB + 1) + c] = r0 + i < N && r0 + c < N ? LU[(r0 + i) * N + r0 + c] : (i == c ? 1.0 : 0.0);
+    __syncthreads();
+    double *v = V + c * (kB + 1);
+    if (!upper) {
+        for (int i = 0; i < kB; ++i) {
+            const double *f = F + i * (kB + 1);
+            double a = i == c ? 1.0 : 0.0, b = 0.0;
+            int q = c;
+            for (; q + 1 < i; q += 2) {
+                a = fma(-f[q], v[q], a);
+                b = fma(-f[q + 1], v[q + 1], b);
+            }
+            if (q < i) a = fma(-f[q], v[q], a);
+            v[i] = i < c ? 0.0 : a + b;
+        }
+    } else {
+        for (int i = kB - 1; i >= 0; --i) {
+            const double *f = F + i * (kB + 1);
+            double a = i == c ? 1.0 : 0.0, b = 0.0;
+            int q = i + 1;
+            for (; q + 1 <= c; q += 2) {
+                a = fma(-f[q], v[q], a);
+                b = fma(-f[q + 1], v[q + 1], b);
+            }
+            if (q <= c) a = fma(-f[q], v[q], a);
+            v[i] = i > c ? 0.0 : (a + b) / f[i];
+        }
+    }
+    __syncthreads();
+    double *o = inv + (2 * j + upper) * kB * kB;
+    for (int q = 0; q < kB; ++q) o[q * kB + c] = V[q * (kB + 1) + c];
+    if (upper ? !(j & 1) : (j & 1)) {  // lower: rows of an odd block, columns before it; upper: the other half
+        const int64_t cb = upper ? r0 + kB : r0 - kB;
+        double *p = off + (2 * (j >> 1) + upper) * kB * kB;
+        __syncthreads();
+        for (int i = 0; i < kB; ++i) F[i * (kB + 1) + c] = r0 + i < N && cb + c < N ? LU[(r0 + i) * N + cb + c] : 0.0;
+        __syncthreads();
+        for (int q = 0; q < kB; ++q) p[q * kB + c] = F[c * (kB + 1) + q];
+    }
+}
+
+// One diagonal block (128 rows from r0) for one right-hand side per thread block: forward x1 =
+// L11^-1 y1, x2 = L22^-1 (y2 - L21 x1), backward the other way round; x replaces y and its digits go
+// to the update. Two threads to a row, each half of the columns.
+__global__ void __launch_bounds__(128) solve_diag(const double *__restrict__ inv, const double *__restrict__ off,
+                                                  int64_t N, int64_t r0, double *__restrict__ Y, int T, int Tp, int upper,
+                                                  unsigned long long *__restrict__ D, int *__restrict__ Ex) {
+    __shared__ double y[2 * kB], part[2 * kB];
+    __shared__ int emax;
+    const int tid = threadIdx.x, i = tid & (kB - 1), h = tid >> 6, t = blockIdx.x;
+    const int64_t b = r0 / kB;
+    if (tid == 0) emax = 0;
+    y[tid] = t < T && r0 + tid < N ? Y[(r0 + tid) * T + t] : 0.0;
+    __syncthreads();
+    auto half_sum = [&](const double *m, const double *v) {  // sum over this thread's half of the columns
+        double a[4] = {};
+#pragma unroll 8
+        for (int q = h * (kB / 2); q < (h + 1) * (kB / 2); q += 4)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a[u] = fma(m[(q + u) * kB + i], v[q + u], a[u]);
+        part[tid] = (a[0] + a[1]) + (a[2] + a[3]);
+        __syncthreads();
+    };
+    const int f = upper ? kB : 0, s = kB - f;  // first and second half in the order of the substitution
+    const int64_t bf = b + (upper ? 1 : 0), bs = b + (upper ? 0 : 1);
+    const bool two = r0 + kB < N;  // the block has a second half
+    if (!upper || two) {
+        half_sum(inv + (2 * bf + upper) * kB * kB, y + f);
+        if (h == 0) y[f + i] = part[i] + part[kB + i];
+        __syncthreads();
+    }
+    if (two) {
+        half_sum(off + (2 * (b >> 1) + upper) * kB * kB, y + f);
+        if (h == 0) y[s + i] -= part[i] + part[kB + i];
+        __syncthreads();
+    }
+    if (two || upper) {
+        half_sum(inv + (2 * bs + upper) * kB * kB, y + s);
+        if (h == 0) y[s + i] = part[i] + part[kB + i];
+        __syncthreads();
+    }
+    const double v = r0 + tid < N ? y[tid] : 0.0;
+    if (t < T && r0 + tid < N) Y[(r0 + tid) * T + t] = v;
+    const int e = __reduce_max_sync(0xffffffffu, exp_field(v));
+    if ((tid & 31) == 0) atomicMax(&emax, e);
+    __syncthreads();
+    const int E = max(emax + 1, kEMin);
+    D[(int64_t)tid * Tp + t] = digits_of(v, E);
+    if (tid == 0) {
+        Ex[t] = E;
+        atomicMax(&Ex[Tp], E);
+    }
+}
+
+__global__ void solve_gather(const double *__restrict__ Q, const int32_t *__restrict__ perm, int64_t N, int T,
+                             double *__restrict__ Y) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= N * T) return;
+    const int64_t i = e / T;
+    Y[e] = Q[(int64_t)perm[i] * T + (e - i * T)];
+}
+
+// out[e] = sum over splits s = 0..S-1 (in that order) of part[s][e], FP64 or an FP32 pair.
+template <typename V>
+__global__ void split_reduce(const double *__restrict__ part, int64_t cnt, int S, V *__restrict__ out) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= cnt) return;
+    double s = part[e];
+    for (int k = 1; k < S; ++k) s += part[k * cnt + e];
+    out[e] = wcast<V>(s);
+}
+
+inline int pad8(int T) { return (T + 7) / 8 * 8; }
+inline size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+struct Plan {
+    int splits;
+    size_t digits, exps, part;
+};
+
+// Splits of the inner dimension: whole rounds of the resident blocks (three per SM), each split as
+// long as possible; half a chunk stands for a block's fixed cost.
+Plan plan(int64_t M, int64_t K, int T, bool direct) {
+    int sms = 152, dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaGetLastError();
+    const int64_t rows = T <= 32 ? 64 : 32, cols = T <= 32 ? 32 : 64, nchunk = (K + kChunk - 1) / kChunk;
+    const int64_t tiles = ((M + rows - 1) / rows) * ((T + cols - 1) / cols);
+    Plan p{1, 0, 0, 0};
+    double best = 1e300;
+    for (int64_t S = 1; S <= 32 && S <= nchunk; ++S) {
+        const int64_t span = (nchunk + S - 1) / S;
+        if ((nchunk + span - 1) / span != S) continue;
+        const int64_t waves = (tiles * S + 3 * sms - 1) / (3 * sms);
+        const double cost = (double)waves * ((double)span + 0.5);
+        if (cost < 0.97 * best) {
+            best = cost;
+            p.splits = (int)S;
+        }
+    }
+    p.digits = up256((size_t)nchunk * kChunk * pad8(T) * 8);
+    p.exps = up256((size_t)nchunk * (pad8(T) + 1) * sizeof(int));
+    p.part = p.splits > 1 || !direct ? (size_t)p.splits * M * T * sizeof(double) : 0;
+    return p;
+}
+
+template <typename Src, typename V, typename O>
+int product(const Src &A, int64_t M, int64_t K, const V *x, int T, O *out, void *ws, cudaStream_t s) {
+    constexpr bool direct = std::is_same<O, double>::value;
+    const Plan p = plan(M, K, T, direct);
+    const int Tp = pad8(T), nchunk = (int)((K + kChunk - 1) / kChunk);
+    unsigned long long *D = (unsigned long long *)ws;
+    int *Ex = (int *)((char *)ws + p.digits);
+    double *part = (double *)((char *)ws + p.digits + p.exps);
+    RBFSL_CUDA_TRY(cudaMemsetAsync(Ex, 0, p.exps, s));
+    x_digits<V><<<dim3((unsigned)nchunk, (unsigned)((Tp + 31) / 32)), 256, 0, s>>>(x, K, T, Tp, D, Ex);
+    const int rc = launch_gemm<Src, V, false>(A, M, K, x, T, Tp, D, Ex, p.splits,
+                                              p.part ? part : reinterpret_cast<double *>(out), s);
+    if (rc || !p.part) return rc;
+    const int64_t cnt = M * T;
+    split_reduce<O><<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(part, cnt, p.splits, out);
+    return launch_status("split product");
+}
+
+}  // namespace
+
+size_t split_product_bytes(int64_t M, int64_t K, int T, int out_dtype) {
+    const Plan p = plan(M, K, T, out_dtype == RBFSL_F64);
+    return p.digits + p.exps + p.part;
+}
+
+int split_apply(const void *E, int64_t M, int64_t K, const void *x, int T, int dtype, void *out, void *ws,
+                cudaStream_t s) {
+    if (dtype == RBFSL_F64)
+        return product(SrcF64{(const double *)E, K}, M, K, (const double *)x, T, (double *)out, ws, s);
+    return product(SrcPair{(const float2 *)E, K}, M, K, (const float2 *)x, T, (float2 *)out, ws, s);
+}
+
+int split_eval(const double *P, int64_t M, const double *X, int64_t K, int kind, double eps, const double *c, int T,
+               int out_dtype, void *out, void *ws, cudaStream_t s) {
+    SrcPhi A{};
+    A.P = P; A.X = X; A.kind = kind; A.eps2 = eps * eps;
+    if (out_dtype == RBFSL_F64) return product(A, M, K, c, T, (double *)out, ws, s);
+    return product(A, M, K, c, T, (float2 *)out, ws, s);
+}
+
+size_t split_solve_factor_bytes(int64_t N) {
+    const int64_t b = (N + kB - 1) / kB;
+    return (size_t)(2 * b + 2 * ((b + 1) / 2)) * kB * kB * sizeof(double);
+}
+
+size_t split_solve_scratch_bytes(int64_t N, int T) {
+    const int64_t b = (N + kChunk - 1) / kChunk;
+    return up256((size_t)kChunk * pad8(T) * 8) + (size_t)2 * b * (pad8(T) + 1) * sizeof(int);
+}
+
+int split_solve_prepare(const double *LU, int64_t N, void *factor, cudaStream_t s) {
+    const int64_t b = (N + kB - 1) / kB;
+    double *inv = (double *)factor, *off = inv + 2 * b * kB * kB;
+    const int smem = 2 * kB * (kB + 1) * (int)sizeof(double);
+    RBFSL_CUDA_TRY(cudaFuncSetAttribute(solve_prepare, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    solve_prepare<<<dim3((unsigned)b, 2), kB, smem, s>>>(LU, N, inv, off);
+    return launch_status("global_solve prepare");
+}
+
+int split_solve(const double *LU, const int32_t *perm, int64_t N, const double *Q, int T, double *C, const void *factor,
+                void *scratch, cudaStream_t s) {
+    const int64_t b64 = (N + kB - 1) / kB, b = (N + kChunk - 1) / kChunk;
+    const double *inv = (const double *)factor, *off = inv + 2 * b64 * kB * kB;
+    const int Tp = pad8(T);
+    unsigned long long *D = (unsigned long long *)scratch;
+    int *Ex = (int *)((char *)scratch + up256((size_t)kChunk * Tp * 8));  // one row per block step
+    RBFSL_CUDA_TRY(cudaMemsetAsync(Ex, 0, (size_t)2 * b * (Tp + 1) * sizeof(int), s));
+    solve_gather<<<(unsigned)((N * T + 255) / 256), 256, 0, s>>>(Q, perm, N, T, C);
+    for (int64_t j = 0; j < 2 * b; ++j) {
+        const int upper = j >= b;
+        const int64_t r0 = (upper ? 2 * b - 1 - j : j) * kChunk, nb = std::min<int64_t>(kChunk, N - r0);
+        int *ex = Ex + j * (Tp + 1);
+        solve_diag<<<(unsigned)Tp, 128, 0, s>>>(inv, off, N, r0, C, T, Tp, upper, D, ex);
+        const int64_t first = upper ? 0 : r0 + nb, rows = upper ? r0 : N - r0 - nb;
+        if (rows <= 0) continue;
+        const SrcF64 A{LU + first * N + r0, N};
+        const int rc = launch_gemm<SrcF64, double, true>(A, rows, nb, C + r0 * T, T, Tp, D, ex, 1, C + first * T, s);
+        if (rc) return rc;
+    }
+    return launch_status("global_solve");
+}
+
+}  // namespace rbfsl
