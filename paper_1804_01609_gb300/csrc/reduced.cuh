@@ -66,18 +66,22 @@ struct RedLayout {
 
 // Stored factors of one centre stencil in the reduced form (doubles): the M x M factor of P1
 // (row-major: R above the diagonal, C below it, 1 / C_kk on it), then W, G = A21 - W A11 (K x M,
-// column-major), W^T (row k of W after the other) and B^-1 (K x K): n^2 + K M doubles, against the
-// (n + M)^2 of an LU factor of the whole system.
+// column-major), W^T (row k of W after the other) and the triangles D^-1 L^-1 and L^-T of B = L D L^T:
+// n^2 + K (M + 1) doubles, against the (n + M)^2 of an LU factor of the whole system.
+// A triangle is folded, row i and row K - 1 - i in one column of K + 1 values, so that lanes along the
+// columns have equal work: entry (i, j), j <= i, at fold(i, j); L^-T with both indexes reversed.
 struct CenterLayout {
-    int W, G, WT, Binv, total;
+    int W, G, WT, T, H, K, total;  // H: columns of a folded triangle
     __host__ __device__ CenterLayout(int n, int M) {
-        const int K = n - M;
+        K = n - M;
+        H = (K + 1) / 2;
         W = M * M;
         G = W + K * M;
         WT = G + K * M;
-        Binv = WT + K * M;
-        total = Binv + K * K;
+        T = WT + K * M;
+        total = T + 2 * H * (K + 1);
     }
+    __host__ __device__ int fold(int i, int j) const { return i < H ? j * H + i : (j + K - i) * H + K - 1 - i; }
 };
 __host__ __device__ inline int center_factor_doubles(int n, int ell, int half) {
     const int M = (ell + 1) * (ell + 1);
@@ -135,9 +139,11 @@ __device__ __forceinline__ bool zero_or_not_finite(double v) {
 // NW gives the same bits. Returns RBFSL_OK with the weights (n doubles, stencil order) in `out`
 // (valid for warp 0), RBFSL_EKNN for a stencil index < 0, RBFSL_ESINGULAR for two coincident
 // stencil nodes, and 1 where a pivot of P or of B vanishes, is not finite or has the wrong sign.
-// kFactor: instead of weights, store the factors that centre stencils keep (CenterLayout) at F and
-// the nodes' pivot order at order (p: any point, its row is not stored).
-template <int NW, bool kTensor, bool kFactor = false>
+// kFactor: instead of weights, store the factors that centre stencils keep (CenterLayout; kFactorCenter)
+// at F and the nodes' pivot order at order (p: any point, its row is not stored). kFactorPatch: L^-1 in the
+// triangles' place (K x K, row-major) and D's diagonal in W^T's (K doubles).
+constexpr int kNoFactor = 0, kFactorCenter = 1, kFactorPatch = 2;
+template <int NW, bool kTensor, int kFactor = kNoFactor>
 __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, const double *__restrict__ X,
                                                      const int32_t *__restrict__ stencil, int n, int M, int ell,
                                                      int half, double px, double py, double pz, int t,
@@ -294,7 +300,7 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
             const int k = e / K, i = e - k * K;
             const double w = P[k * S + M + i];
             F[fl.W + e] = w;
-            F[fl.WT + i * M + k] = w;
+            if (kFactor == kFactorCenter) F[fl.WT + i * M + k] = w;
         }
         for (int i = t; i < n; i += GT) order[i] = ord[i];
         if (kTensor) gsync();
@@ -488,21 +494,29 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
         gsync();
     }
     if (kFactor) {
-        // ---- B^-1 = L^-T D^-1 L^-1, a thread per column, in place in global memory
+        // ---- L^-1, a thread per column, in place in global memory
+        double *T1 = F + fl.T, *T2 = T1 + fl.H * (K + 1);
         for (int c = t; c < K; c += GT) {
-            double *x = F + fl.Binv + c;  // x_i at x[i * K]
+            auto at = [&](int i) { return kFactor == kFactorPatch ? i * K + c : fl.fold(i, c); };
             for (int i = 0; i < K; ++i) {
                 const double *li = B + tri(i);
+                if (i < c) {
+                    if (kFactor == kFactorPatch) T1[at(i)] = 0.0;
+                    continue;
+                }
                 double a = i == c ? 1.0 : 0.0;
-                for (int j = c; j < i; ++j) a = fma(-li[j], x[j * K], a);
-                x[i * K] = i < c ? 0.0 : a;
+                for (int j = c; j < i; ++j) a = fma(-li[j], T1[at(j)], a);
+                T1[at(i)] = a;
+                if (kFactor == kFactorCenter) T2[fl.fold(K - 1 - c, K - 1 - i)] = a;
             }
-            for (int i = K - 1; i >= 0; --i) {
-                double a = i < c ? 0.0 : x[i * K] / B[tri(i) + i];
-                for (int j = i + 1; j < K; ++j) a = fma(-B[tri(j) + i], x[j * K], a);
-                x[i * K] = a;
+            if (kFactor == kFactorPatch) {
+                F[fl.WT + c] = B[tri(c) + c];
+                continue;
             }
+            for (int i = c; i < K; ++i) T1[at(i)] /= B[tri(i) + i];
         }
+        if (kFactor == kFactorCenter && (K & 1))  // the middle row has a column to itself
+            for (int e = fl.H + t; e <= K; e += GT) T1[e * fl.H + fl.H - 1] = T2[e * fl.H + fl.H - 1] = 0.0;
         return RBFSL_OK;
     }
     if (warp != 0) return RBFSL_OK;
@@ -551,16 +565,18 @@ __device__ __forceinline__ int weights_point(double *__restrict__ R, const doubl
 
 // ---- Centre stencils (Sec. 3.3): the point uses the stencil of its nearest node, whose reduced
 // factors are kept. Per point u = P1^-T Y(p) by substitution with P1's factor, g = phi_2 - W phi_1 -
-// G u, w2 = B^-1 g and w1 = u - W^T w2: the last form keeps the weights' polynomial part exact
-// whatever the rounding of w2, so the inverse of B serves as well as its factors, and the three
-// products run without a serial chain. kLanes lanes of a warp per point.
+// G u, w2 = L^-T (D^-1 L^-1 g) and w1 = u - W^T w2: the last form keeps the weights' polynomial part exact
+// whatever the rounding of w2, and the products run without a serial chain across lanes. The inverse of
+// B itself, one product of the same size, does not serve: on coarse node sets, where g is small against
+// |B| |B^-1| |g|, its weights lost two digits (N = 642, n = 84: 2e-12 against 5e-14 for LU factors; the
+// triangles 5e-14). kLanes lanes of a warp per point.
 //
 // Bound: the FP64 pipe (two thirds of the multiplications of substituting through an LU factor of
-// the whole system, and a serial chain of 2 M steps instead of 2 (n + M)), then HBM (8 (n^2 + K M)
-// bytes per point). N = 40,962, n = 84 1.16 ms against 2.33 ms, N = 163,842, n = 31 0.91 ms against
+// the whole system, and a serial chain of 2 M steps instead of 2 (n + M)), then HBM (8 (n^2 + K (M + 1))
+// bytes per point). N = 40,962, n = 84 1.15 ms against 2.33 ms, N = 163,842, n = 31 0.90 ms against
 // 1.91 ms for the LU factors, which stay for the systems without the reduced form.
 
-// Shared doubles of one point: P1's factor, phi (later w2), Y(p), u, g and the weights.
+// Shared doubles of one point: P1's factor, phi (later z = D^-1 L^-1 g), Y(p), u, g (later w2) and the weights.
 __host__ __device__ inline int center_reduced_doubles(int n, int M) { return M * M + 3 * n + M; }
 
 // Lanes per point: half a warp where the products then leave fewer lanes idle (K <= 32, M <= 16:
@@ -608,22 +624,31 @@ __device__ __forceinline__ double *center_point_reduced(const double *__restrict
         g[i] = a0 + a1;
     }
     __syncwarp();
-    for (int i = l; i < K; i += kLanes) {
-        const double *b = F + fl.Binv + i;
-        double a0 = 0.0, a1 = 0.0;
-        int j = 0;
+    // a folded triangle times x, two rows a lane: out(row, value)
+    auto triangle = [&](const double *tr, auto x, auto out) {
+        for (int c = l; c < fl.H; c += kLanes) {
+            const double *p = tr + c;
+            double a = 0.0, first = 0.0;
 #pragma unroll 8
-        for (; j + 1 < K; j += 2) {
-            a0 = fma(b[j * K], g[j], a0);
-            a1 = fma(b[(j + 1) * K], g[j + 1], a1);
+            for (int e = 0; e <= K; ++e) {
+                a = fma(p[e * fl.H], x(e <= c ? e : e - c - 1), a);
+                if (e == c) {
+                    first = a;
+                    a = 0.0;
+                }
+            }
+            out(c, first);
+            if (K - 1 - c != c) out(K - 1 - c, a);
         }
-        if (j < K) a0 = fma(b[j * K], g[j], a0);
-        phi[M + i] = a0 + a1;
-        out[order[M + i]] = a0 + a1;
-    }
-    __syncwarp();
+        __syncwarp();
+    };
+    triangle(F + fl.T, [&](int j) { return g[j]; }, [&](int i, double v) { phi[M + i] = v; });
+    triangle(F + fl.T + fl.H * (K + 1), [&](int j) { return phi[M + K - 1 - j]; }, [&](int i, double v) {
+        g[K - 1 - i] = v;
+        out[order[M + K - 1 - i]] = v;
+    });
     for (int k = l; k < M; k += kLanes) {
-        const double *w = F + fl.WT + k, *z = phi + M;
+        const double *w = F + fl.WT + k, *z = g;
         double a0 = u[k], a1 = 0.0;
         int i = 0;
 #pragma unroll 8

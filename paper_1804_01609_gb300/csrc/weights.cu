@@ -192,9 +192,9 @@ __global__ void __launch_bounds__(128, 4) center_factor_kernel(const double *__r
     const int64_t c = s0 < 0 ? 0 : s0;
     const int t = threadIdx.x;
     const int rc = reduced_on_tensor(M)
-                       ? weights_point_reduced<4, true, true>(sm, X, Ik + k * n, n, M, ell, half, X[3 * c], X[3 * c + 1],
+                       ? weights_point_reduced<4, true, kFactorCenter>(sm, X, Ik + k * n, n, M, ell, half, X[3 * c], X[3 * c + 1],
                                                               X[3 * c + 2], t, out, Fk, order + (size_t)k * n)
-                       : weights_point_reduced<4, false, true>(sm, X, Ik + k * n, n, M, ell, half, X[3 * c], X[3 * c + 1],
+                       : weights_point_reduced<4, false, kFactorCenter>(sm, X, Ik + k * n, n, M, ell, half, X[3 * c], X[3 * c + 1],
                                                                X[3 * c + 2], t, out, Fk, order + (size_t)k * n);
     if (t == 0 && rc != RBFSL_OK) atomicAdd(&bad[rc == RBFSL_EKNN ? 1 : 0], 1);
 }

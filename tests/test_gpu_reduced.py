@@ -80,3 +80,32 @@ def test_centre_stencils_match_oracle(orc, n, ell, p, prec):
     ref = orc.local_run(X, q, n, ell, p, rbfsl.VEL_DEFORM_Y2, vp, dt, steps, mode=orc.CENTER)
     exact = _parity.exact_field(fields, X, rbfsl.VEL_DEFORM_Y2, vp, steps * dt)
     _parity.check_run(f"centre n={n} ell={ell} r^{p} prec={prec}", got, ref, exact, strict=False)
+
+
+# coarse node sets, where the reduced matrix is worst conditioned: one step at the oracle's noise floor
+# (its change when every coordinate moves by one ulp; five times it, plus 1e-12 of max|q|)
+@pytest.mark.parametrize("N,n,ell,p", [(642, 84, 4, 9), (900, 84, 4, 9), (642, 55, 3, 7), (642, 31, 2, 5)])
+def test_centre_stencils_on_coarse_nodes(orc, N, n, ell, p):
+    X = inputs.nodes(N, 11)
+    vp = inputs.nl_deformation_params(5.0)
+    rng = np.random.default_rng(N)
+    q = np.stack([inputs.plane_wave_field(rng, 6.0)(X) for _ in range(3)], axis=1)
+
+    def reference(Y):
+        return orc.local_run(Y, q, n, ell, p, rbfsl.VEL_NL, vp, 0.1, 1, mode=orc.CENTER)
+
+    ref = reference(X)
+    floor = np.abs(reference(np.nextafter(X, X + rng.choice([-1.0, 1.0], size=X.shape))) - ref).max()
+    c = rbfsl.Context(0)
+    c.set_nodes(X)
+    c.set_velocity(rbfsl.VEL_NL, vp)
+    c.set_method(rbfsl.LOCAL, rbfsl.CENTER)
+    c.set_stencil_size(n)
+    c.set_sh_degree(ell)
+    c.set_kernel(rbfsl.PHS, p)
+    c.set_dt(0.1)
+    c.set_tracers(q)
+    c.step(1)
+    err = np.abs(c.get_q() - ref).max()
+    c.close()
+    assert err <= 5 * floor + 1e-12 * np.abs(q).max()
