@@ -227,7 +227,8 @@ int rbfsl_global_eval(const double *p, int64_t Nq, const double *x, int64_t N, i
  * around Mp given centres (the paper takes R = 2 sqrt(n / N) for ~n nodes per patch,
  * Eq. rad_patches, and Mp = ceil(a N / n) centres, Eq. num_patches). Creation finds each
  * patch's nodes, assembles its augmented PHS + spherical-harmonic system (Eq.
- * rbf_poly_linsys, degree ell) and factorises it once (LU with partial pivoting, FP64).
+ * rbf_poly_linsys, degree ell) and factorises it once in FP64 (reduced to the null space of the
+ * harmonics; LU with partial pivoting where a patch has no reduced form).
  *   x: device N x 3, centers: device Mp x 3 (copied). kernel must be RBFSL_PHS with odd p.
  *   Synchronises `stream`. Errors: EINVAL (a patch with no node, or more than
  *   RBFSL_MAX_SYSTEM - (ell+1)^2 nodes), ESINGULAR, ENOMEM, ECUDA. */
@@ -245,7 +246,8 @@ int rbfsl_pu_destroy(rbfsl_pu *pu);
  * evaluation; RBFSL_F32: FP32 evaluation, out FP32; RBFSL_F32X2: each term's factor formed in
  * FP64, coefficients and sums as FP32 pairs (hi, lo) in pair arithmetic, out N x T pairs
  * (~n 2^-48 relative rounding, against the patch sums' cancellation). The handle keeps a coefficient buffer
- * (reallocated when T changes), so calls on one handle must not overlap.
+ * (reallocated when T changes) and a stream of its own, joined to `stream` before the call's last
+ * kernels, so calls on one handle must not overlap.
  * status: device Nq or NULL (RBFSL_EUNCOVERED for a point in no patch, RBFSL_EINVAL for a
  * point in more than 32 patches; out row NaN). Errors: EINVAL, ENOMEM, ECUDA. */
 int rbfsl_pu_apply(rbfsl_pu *pu, const double *q, int T, const double *p, int64_t Nq,

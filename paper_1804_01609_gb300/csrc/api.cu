@@ -310,12 +310,12 @@ int one_step_global(rbfsl_ctx *c) {
     return RBFSL_OK;
 }
 
-// RBF-PU (Sec. 3.3): patches and their LU factors once; per step the patch coefficients and
+// RBF-PU (Sec. 3.3): patches and their factors once; per step the patch coefficients and
 // the blended evaluation at the departure points.
 int prepare_pu(rbfsl_ctx *c) {
     if (!c->pu_centers) return fail(c, RBFSL_ENOTCONF, "set_pu has not been called");
     if (c->kkind != RBFSL_PHS) return fail(c, RBFSL_EINVAL, "the RBF-PU method needs the PHS kernel");
-    const int64_t N = c->N, T = c->T;
+    const int64_t N = c->N;
     double R = c->pu_radius;
     if (!(R > 0)) {
         if (c->n < 1) return fail(c, RBFSL_ENOTCONF, "RBF-PU radius needs a stencil size (nodes per patch)");
@@ -327,9 +327,6 @@ int prepare_pu(rbfsl_ctx *c) {
     if ((rc = dalloc(c, &c->status, N * sizeof(int32_t)))) return rc;
     if ((rc = dalloc(c, &c->ctr, 3 * sizeof(unsigned long long)))) return rc;
     CTX_TRY(c, cudaMemsetAsync(c->ctr, 0, 3 * sizeof(unsigned long long), c->stream));
-    if (c->precision == RBFSL_MIXED) {
-        if ((rc = dalloc(c, &c->Q64, N * T * sizeof(double)))) return rc;
-    }
     CTX_RC(c, rbfsl_pu_create(&c->pu, c->X, N, c->pu_centers, c->pu_Mp, R, ell, c->kkind, c->kparam, c->stream));
     c->bytes += c->pu->bytes;
     c->prepared_T = c->T;
@@ -338,19 +335,15 @@ int prepare_pu(rbfsl_ctx *c) {
 }
 
 int one_step_pu(rbfsl_ctx *c) {
-    const int64_t N = c->N, NT = N * (int64_t)c->T;
+    const int64_t N = c->N;
     const double t1 = c->t + c->dt;
-    CTX_RC(c, launch_trace_order(c->X, N, c->vel_kind, c->vel, t1, c->dt, c->precision, c->integrator, c->xi, c->stream));
-    const double *q64 = (const double *)c->q;
-    const unsigned blocks = (unsigned)((NT + 255) / 256);
-    if (c->precision == RBFSL_MIXED) {
-        from_pair_kernel<double><<<blocks, 256, 0, c->stream>>>((const float2 *)c->q, c->Q64, NT);
-        q64 = c->Q64;
-    }
-    // mixed: FP64 coefficient solves, the blend in FP32-pair arithmetic straight into the pair field
-    CTX_RC(c, rbfsl_pu_apply(c->pu, q64, c->T, c->xi, N, c->pu_wkind,
-                             c->precision == RBFSL_FP64 ? RBFSL_F64 : RBFSL_F32X2, c->q_next, c->status,
-                             c->stream));
+    // mixed: FP64 coefficients, the blend in FP32-pair arithmetic straight into the pair field. The
+    // coefficients do not depend on the departure points.
+    const int dtype = c->precision == RBFSL_FP64 ? RBFSL_F64 : RBFSL_F32X2;
+    CTX_RC(c, pu_apply_begin(c->pu, c->q, dtype, c->T, dtype, c->stream));
+    const int rc = launch_trace_order(c->X, N, c->vel_kind, c->vel, t1, c->dt, c->precision, c->integrator, c->xi, c->stream);
+    CTX_RC(c, pu_apply_end(c->pu, c->T, c->xi, N, c->pu_wkind, dtype, c->q_next, c->status, c->stream));
+    CTX_RC(c, rc);
     count_status<<<(unsigned)((N + 255) / 256), 256, 0, c->stream>>>(c->status, N, c->ctr);
     std::swap(c->q, c->q_next);
     c->t = t1;

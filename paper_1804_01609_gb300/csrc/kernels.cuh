@@ -24,14 +24,21 @@ struct rbfsl_pu {
     double *X = nullptr, *centers = nullptr;
     int64_t *mstart = nullptr;   // Mp + 1 (device)
     int32_t *members = nullptr;  // mstart[Mp] (device), ascending node index per patch
-    int64_t *lu_off = nullptr;   // Mp (device): offset of patch l's m_l x m_l factor
+    int reduced = 0;             // 1: reduced factors as digits (PatchLayout), 0: LU factors
+    int64_t *lu_off = nullptr;   // Mp (device): offset of patch l's factors
     double *LU = nullptr;
-    int32_t *perm = nullptr;     // row order of each factor, at mstart[l] + l * M
+    int32_t *perm = nullptr;     // pivot (reduced) or row (LU) order, at mstart[l] + l * M
+    int32_t *pmem = nullptr;     // reduced: members in pivot order, at mstart[l]
+    double *mx = nullptr;        // members' coordinates, patch l's from row mstart[l] + l M on
     rbfsl_knn_index *nodes_ix = nullptr, *centers_ix = nullptr;
-    double *coef = nullptr;      // (mstart[Mp] + Mp M) x coef_T
-    void *coef32 = nullptr;      // FP32 or FP32-pair copy of coef for the mixed evaluations
+    void *coef = nullptr;        // (mstart[Mp] + Mp M) x coef_T values of 8 bytes at most
     int coef_T = 0;
-    int64_t coef_len = 0;        // values in coef
+    int64_t rows = 0;            // mstart[Mp] + Mp M
+    int64_t chunk = 0;           // points per launch of the blend, and their patches and harmonics
+    int32_t *pt_cnt = nullptr, *pt_id = nullptr;
+    double *pt_w = nullptr, *pt_Y = nullptr;
+    cudaStream_t side = nullptr;  // the coefficients, beside the tracing and the points' patches
+    cudaEvent_t fork = nullptr, join = nullptr;
     int32_t *status = nullptr;
     size_t bytes = 0;
 };
@@ -114,6 +121,47 @@ __device__ __forceinline__ void grid_ball_foreach(const KnnGrid &g, double qx, d
     }
 }
 
+// The same for one thread: f(p) for the sorted positions p of the cells that the ball touches.
+template <typename F>
+__device__ __forceinline__ void grid_ball_rows(const KnnGrid &g, double qx, double qy, double qz, double rb, F f) {
+    const float x = (float)qx, y = (float)qy, z = (float)qz, r = (float)rb * 1.00001f + 1e-6f;
+    const float inv = (float)g.inv_cell, edge = 1.0f / inv;
+    const int G = g.G;
+    auto cell = [&](float v, float margin) {
+        const int c = (int)floorf((v + 1.0f) * inv + margin);
+        return c < 0 ? 0 : (c >= G ? G - 1 : c);
+    };
+    auto outside = [&](float v, int c) {
+        const float lo = c == 0 ? -1e30f : c * edge - 1.0f, hi = c == G - 1 ? 1e30f : (c + 1) * edge - 1.0f;
+        return fmaxf(fmaxf(lo - v, v - hi), 0.0f);
+    };
+    const int y0 = cell(y - r, -1e-3f), y1 = cell(y + r, 1e-3f), z0 = cell(z - r, -1e-3f), z1 = cell(z + r, 1e-3f);
+    // four rows' ranges are loaded together: a thread by itself waits for each of its loads
+    const int ny = y1 - y0 + 1, rows = ny * (z1 - z0 + 1);
+    int cy = y0, cz = z0;
+    for (int base = 0; base < rows; base += 4) {
+        int b[4], e[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            b[u] = e[u] = 0;
+            const float dy = outside(y, cy), dz = outside(z, cz), h2 = r * r - dy * dy - dz * dz;
+            if (base + u < rows && h2 >= -1e-4f * r * r) {
+                const float h = sqrtf(fmaxf(h2, 0.0f)) * 1.00001f + 0.02f * r;
+                const int64_t c = (int64_t)(cz * G + cy) * G;
+                b[u] = g.cell_start[c + cell(x - h, -1e-3f)];
+                e[u] = g.cell_start[c + cell(x + h, 1e-3f) + 1];
+            }
+            if (++cy > y1) {
+                cy = y0;
+                ++cz;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            for (int p = b[u]; p < e[u]; ++p) f(p);
+    }
+}
+
 int launch_trace(const double *x, int64_t N, int vel_kind, const double *prm, double t1,
                  double dt, int precision, double *xi, cudaStream_t s);
 
@@ -132,6 +180,13 @@ int launch_gather(const int32_t *idx, const void *w, int64_t Nq, int n, const vo
                   int dtype, void *q_out, cudaStream_t s);
 
 int sh_tables_init();
+
+// rbfsl_pu_apply in two parts. begin: the coefficients of a field of q_dtype (RBFSL_F64, or RBFSL_F32X2: FP32
+// pairs) on the handle's side stream, after what is on s; end (also after an error in between): the points'
+// patches on s, then, with the coefficients there, the blend. q must stay unchanged until end's work on s.
+int pu_apply_begin(rbfsl_pu *u, const void *q, int q_dtype, int T, int dtype, cudaStream_t s);
+int pu_apply_end(rbfsl_pu *u, int T, const double *p, int64_t Nq, int wkind, int dtype, void *out, int32_t *status,
+                 cudaStream_t s);
 
 int launch_stencil_factor(const double *X, const int64_t *mstart, const int32_t *members,
                           const int64_t *lu_off, int64_t count, int max_n, int M, int ell,

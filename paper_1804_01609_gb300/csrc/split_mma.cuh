@@ -57,20 +57,36 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], c
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
+// The digits of a lane's part of B (16 x 8): rows t, t + 1, t + 8 and t + 9 of its column as FP16 pairs.
+__device__ __forceinline__ void digit_frags(uint32_t (&b)[kDigits][2], unsigned long long b0, unsigned long long b1,
+                                            unsigned long long b2, unsigned long long b3) {
+#pragma unroll
+    for (int s = 0; s < kDigits; ++s) {
+        b[s][0] = digit_pair(b0, b1, s);
+        b[s][1] = digit_pair(b2, b3, s);
+    }
+}
+
+// acc[g] += the digit products of weight g of a lane's part of A (16 x 16; x[4 u + v]: row g + 8 u,
+// columns t, t + 1, t + 8, t + 9) and of B.
+__device__ __forceinline__ void split_products(float (&acc)[kGroups][4], const unsigned long long (&x)[8],
+                                               const uint32_t (&b)[kDigits][2]) {
+#pragma unroll
+    for (int s = 0; s < kDigits; ++s) {
+        const uint32_t a[4] = {digit_pair(x[0], x[1], s), digit_pair(x[4], x[5], s), digit_pair(x[2], x[3], s),
+                               digit_pair(x[6], x[7], s)};
+#pragma unroll
+        for (int q = 0; q < kDigits && s + q < kGroups; ++q) mma_f16(acc[s + q], a, b[q]);
+    }
+}
+
 // acc[g] += the digit products of weight g of A (16 x 16) and B (16 x 8), one warp. A(r, k) for
 // r in {g, g + 8}, B(k): this lane's column; both return digits_of a number (0x8080...: zero).
 template <typename FA, typename FB>
 __device__ __forceinline__ void split_mma(float (&acc)[kGroups][4], int lane, FA A, FB B) {
     const int g = lane >> 2, t = (lane & 3) * 2;
     uint32_t b[kDigits][2];
-    {
-        const unsigned long long b0 = B(t), b1 = B(t + 1), b2 = B(t + 8), b3 = B(t + 9);
-#pragma unroll
-        for (int s = 0; s < kDigits; ++s) {
-            b[s][0] = digit_pair(b0, b1, s);
-            b[s][1] = digit_pair(b2, b3, s);
-        }
-    }
+    digit_frags(b, B(t), B(t + 1), B(t + 8), B(t + 9));
     unsigned long long x[8];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -81,13 +97,7 @@ __device__ __forceinline__ void split_mma(float (&acc)[kGroups][4], int lane, FA
         x[4 * u + 3] = A(r, t + 9);
     }
     __syncwarp();
-#pragma unroll
-    for (int s = 0; s < kDigits; ++s) {
-        const uint32_t a[4] = {digit_pair(x[0], x[1], s), digit_pair(x[4], x[5], s), digit_pair(x[2], x[3], s),
-                               digit_pair(x[6], x[7], s)};
-#pragma unroll
-        for (int q = 0; q < kDigits && s + q < kGroups; ++q) mma_f16(acc[s + q], a, b[q]);
-    }
+    split_products(acc, x, b);
 }
 
 // An integer below 2^51 in magnitude as a double (one FP64 addition).
