@@ -263,7 +263,6 @@ struct PatchLayout {
     }
 };
 
-constexpr unsigned long long kZeroDigits = 0x8080808080808080ULL;
 constexpr int kPuTracers = 16;  // tracers per block
 // the sums of digit products stay below 2^24: at most seven products of full digits (2^14) per weight
 // beside two with a leading digit (|digit| <= 32)

@@ -124,8 +124,14 @@ __device__ __forceinline__ double chunk_scale(int EA, int EX) {
     return __longlong_as_double((long long)(e > 0 ? e : 0) << 52);
 }
 
-// kSub: C[r][t] -= sum; else to out (row length T) + split * M * T.
-template <typename Src, typename V, int kWarpRows, bool kSub>
+// Whether a chunk's sums need plain FP64: rows (2 kENan) or columns that are not finite, or results beyond
+// the doubles' range.
+__device__ __forceinline__ bool chunk_bad(int ea_max, int ex_max) {
+    return ea_max > kENan || ex_max > kENan || ea_max + ex_max >= 2047 + 1023 + 34;
+}
+
+// To out (row length T) + split * M * T.
+template <typename Src, typename V, int kWarpRows>
 __global__ void __launch_bounds__(128, 3) split_gemm_kernel(Src A, int64_t M, int64_t K, const V *__restrict__ x, int T,
                                                             int Tp, const unsigned long long *__restrict__ D,
                                                             const int *__restrict__ Ex, int nchunk, int span,
@@ -164,7 +170,7 @@ __global__ void __launch_bounds__(128, 3) split_gemm_kernel(Src A, int64_t M, in
                 e = __reduce_max_sync(0xffffffffu, e);
                 const int E = max(e + 1, kEMin);
                 if (lane == 0) Er[row] = E;
-                bad |= e >= kENan || exm > kENan || E + exm >= 2047 + 1023 + 34;
+                bad |= chunk_bad(e >= kENan ? 2 * kENan : E, exm);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) As[row * kLd + lane + 32 * u] = Src::digits(w[v][u], E);
             }
@@ -241,12 +247,11 @@ __global__ void __launch_bounds__(128, 3) split_gemm_kernel(Src A, int64_t M, in
             const int64_t r = r0 + wr + g + 8 * (u >> 1);
             const int t = col0 + 8 * nt + t2 + (u & 1);
             if (r >= M || t >= T) continue;
-            if (kSub) out[r * T + t] -= sum[nt][u];
-            else out[((int64_t)blockIdx.z * M + r) * T + t] = sum[nt][u];
+            out[((int64_t)blockIdx.z * M + r) * T + t] = sum[nt][u];
         }
 }
 
-template <typename Src, typename V, bool kSub>
+template <typename Src, typename V>
 int launch_gemm(const Src &A, int64_t M, int64_t K, const V *x, int T, int Tp, const unsigned long long *D, const int *Ex,
                 int splits, double *out, cudaStream_t s) {
     const int nchunk = (int)((K + kChunk - 1) / kChunk), span = (nchunk + splits - 1) / splits;
@@ -256,13 +261,36 @@ int launch_gemm(const Src &A, int64_t M, int64_t K, const V *x, int T, int Tp, c
         dim3 grid((unsigned)((M + rows - 1) / rows), (unsigned)((T + cols - 1) / cols), (unsigned)splits);
         kernel<<<grid, 128, smem, s>>>(A, M, K, x, T, Tp, D, Ex, nchunk, span, out);
     };
-    if (T <= 32) go(split_gemm_kernel<Src, V, 4, kSub>, 64, 32);
-    else go(split_gemm_kernel<Src, V, 2, kSub>, 32, 64);
+    if (T <= 32) go(split_gemm_kernel<Src, V, 4>, 64, 32);
+    else go(split_gemm_kernel<Src, V, 2>, 32, 64);
     return launch_status("split_gemm");
 }
 
 // ---- triangular solves with diagonal blocks of 128 rows
 constexpr int kB = 64;  // inverted triangular blocks (two to a diagonal block)
+
+// Programmatic dependent launch: the next kernel of the stream may start (its prologue runs beside this
+// kernel), and wait until every kernel before this one is complete. What an earlier kernel of the chain
+// wrote is read through pointers without __restrict__: loads that the compiler takes for invariant could
+// move ahead of the wait.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_dependencies() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// A launch whose blocks may start beside the kernel before it in the stream (they wait in the kernel).
+template <typename... P, typename... A>
+void launch_after_prologue(void (*kernel)(P...), dim3 grid, int threads, int smem, cudaStream_t s, A... a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(a)...);  // errors: launch_status of the caller
+}
 
 // Inverses of the 64 x 64 diagonal blocks of the unit lower (blockIdx.y = 0) and the upper factor
 // (1), column-major, and the 64 x 64 block that couples a diagonal block's halves (also
@@ -318,41 +346,54 @@ __global__ void __launch_bounds__(64) solve_prepare(const double *__restrict__ L
 
 // One diagonal block (128 rows from r0) for one right-hand side per thread block: forward x1 =
 // L11^-1 y1, x2 = L22^-1 (y2 - L21 x1), backward the other way round; x replaces y and its digits go
-// to the update. Two threads to a row, each half of the columns.
+// to the update. Two threads to a row, each half of the columns. Bound: latency; a thread's 96 matrix
+// entries are loaded beside the kernel before (the columns of the padding, and those of a missing second
+// half, are the identity's).
 __global__ void __launch_bounds__(128) solve_diag(const double *__restrict__ inv, const double *__restrict__ off,
-                                                  int64_t N, int64_t r0, double *__restrict__ Y, int T, int Tp, int upper,
-                                                  unsigned long long *__restrict__ D, int *__restrict__ Ex) {
+                                                  int64_t N, int64_t r0, double *Y, int T, int Tp, int upper,
+                                                  unsigned long long *D, int *Ex) {
     __shared__ double y[2 * kB], part[2 * kB];
     __shared__ int emax;
     const int tid = threadIdx.x, i = tid & (kB - 1), h = tid >> 6, t = blockIdx.x;
     const int64_t b = r0 / kB;
-    if (tid == 0) emax = 0;
-    y[tid] = t < T && r0 + tid < N ? Y[(r0 + tid) * T + t] : 0.0;
-    __syncthreads();
-    auto half_sum = [&](const double *m, const double *v) {  // sum over this thread's half of the columns
-        double a[4] = {};
-#pragma unroll 8
-        for (int q = h * (kB / 2); q < (h + 1) * (kB / 2); q += 4)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) a[u] = fma(m[(q + u) * kB + i], v[q + u], a[u]);
-        part[tid] = (a[0] + a[1]) + (a[2] + a[3]);
-        __syncthreads();
-    };
     const int f = upper ? kB : 0, s = kB - f;  // first and second half in the order of the substitution
     const int64_t bf = b + (upper ? 1 : 0), bs = b + (upper ? 0 : 1);
     const bool two = r0 + kB < N;  // the block has a second half
+    launch_dependents();
+    constexpr int kH = kB / 2;
+    double m1[kH], m2[kH], m3[kH];
+    auto load = [&](double(&m)[kH], bool on, const double *p) {
+#pragma unroll
+        for (int q = 0; q < kH; ++q) m[q] = on ? p[(h * kH + q) * kB + i] : 0.0;
+    };
+    load(m1, !upper || two, inv + (2 * bf + upper) * kB * kB);
+    load(m2, two, off + (2 * (b >> 1) + upper) * kB * kB);
+    load(m3, two || upper, inv + (2 * bs + upper) * kB * kB);
+    if (tid == 0) emax = 0;
+    wait_dependencies();
+    y[tid] = t < T && r0 + tid < N ? Y[(r0 + tid) * T + t] : 0.0;
+    __syncthreads();
+    auto half_sum = [&](const double(&m)[kH], const double *v) {  // sum over this thread's half of the columns
+        double a[4] = {};
+#pragma unroll
+        for (int q = 0; q < kH; q += 4)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a[u] = fma(m[q + u], v[h * kH + q + u], a[u]);
+        part[tid] = (a[0] + a[1]) + (a[2] + a[3]);
+        __syncthreads();
+    };
     if (!upper || two) {
-        half_sum(inv + (2 * bf + upper) * kB * kB, y + f);
+        half_sum(m1, y + f);
         if (h == 0) y[f + i] = part[i] + part[kB + i];
         __syncthreads();
     }
     if (two) {
-        half_sum(off + (2 * (b >> 1) + upper) * kB * kB, y + f);
+        half_sum(m2, y + f);
         if (h == 0) y[s + i] -= part[i] + part[kB + i];
         __syncthreads();
     }
     if (two || upper) {
-        half_sum(inv + (2 * bs + upper) * kB * kB, y + s);
+        half_sum(m3, y + s);
         if (h == 0) y[s + i] = part[i] + part[kB + i];
         __syncthreads();
     }
@@ -367,6 +408,129 @@ __global__ void __launch_bounds__(128) solve_diag(const double *__restrict__ inv
         Ex[t] = E;
         atomicMax(&Ex[Tp], E);
     }
+}
+
+// The solve's update C[r][t] -= sum over k < kc of A[r][k] x[k][t], 16 rows and 64 / KW columns a block:
+// KW warps along k and 4 / KW along the columns (16 each). One launch of a chain of 2 N / 128, each
+// waiting for the one before: few rows a block, the factor's digits formed beside the kernel before, and,
+// where that leaves SMs idle, the inner dimension split over the warps (launch_update). N = 4,999, T = 9, a step (80 links, evaluation
+// 0.83 ms): 64-row blocks with a warp's whole inner dimension, each link after the one before 3.30 ms, now
+// 1.87; N = 10,242, T = 64 (160 links) 7.37 ms, with prologues beside the link before 6.89, now 4.20.
+constexpr int64_t kUpdateBlocks = 4 * 152;
+
+template <int KW>
+__global__ void __launch_bounds__(128, 3) solve_update(SrcF64 A, int64_t M, int kc, const double *x, int T, int Tp,
+                                                       const unsigned long long *D, const int *Ex, double *C) {
+    constexpr int CW = 4 / KW, kCols = 16 * CW, kSteps = 8 / KW;
+    __shared__ __align__(16) unsigned long long As[16 * kLd];
+    __shared__ double part[KW][16 * kCols];
+    __shared__ int Er[16];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t2 = (lane & 3) * 2;
+    const int64_t r0 = (int64_t)blockIdx.x * 16;
+    const int col0 = blockIdx.y * kCols;
+    launch_dependents();
+    int ea_max = 0;
+    {
+        unsigned long long w[4][4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t r = r0 + 4 * warp + v;
+                const int k = lane + 32 * u;
+                w[v][u] = r < M && k < kc ? A.raw(r, k) : 0ULL;
+            }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            int e = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) e = max(e, SrcF64::field(w[v][u]));
+            e = __reduce_max_sync(0xffffffffu, e);
+            const int E = max(e + 1, kEMin);
+            if (lane == 0) Er[4 * warp + v] = E;
+            ea_max = max(ea_max, e >= kENan ? 2 * kENan : E);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) As[(4 * warp + v) * kLd + lane + 32 * u] = SrcF64::digits(w[v][u], E);
+        }
+    }
+    wait_dependencies();
+    const int kw = warp / CW, cb = col0 + 16 * (warp % CW);
+    const bool on = cb < Tp, two = cb + 8 < Tp;
+    unsigned long long nx[2][2][4];  // x's digits (D has 128 rows, zeros behind kc), a step ahead
+    auto load = [&](int q, unsigned long long(&d)[2][4]) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                d[h][v] = on && (h == 0 || two)
+                              ? D[(int64_t)((kw * kSteps + q) * 16 + t2 + (v & 1) + 8 * (v >> 1)) * Tp + cb + 8 * h + g]
+                              : kZeroDigits;
+    };
+    load(0, nx[0]);
+    constexpr int kOut = 16 * kCols / 128;  // outputs of a thread: row, then column
+    double old[kOut];
+#pragma unroll
+    for (int o = 0; o < kOut; ++o) {
+        const int e = threadIdx.x + 128 * o, r = e / kCols, t = col0 + e % kCols;
+        old[o] = r0 + r < M && t < T ? C[(r0 + r) * T + t] : 0.0;
+    }
+    const bool bad = __syncthreads_or(chunk_bad(ea_max, Ex[Tp]));
+    if (!bad && on) {
+        float acc[2][kGroups][4] = {};
+#pragma unroll
+        for (int q = 0; q < kSteps; ++q) {
+            if (q + 1 < kSteps) load(q + 1, nx[(q + 1) & 1]);
+            const unsigned long long *a = As + g * kLd + (kw * kSteps + q) * 16 + t2;
+            const ulonglong2 a0 = *reinterpret_cast<const ulonglong2 *>(a),
+                             a1 = *reinterpret_cast<const ulonglong2 *>(a + 8),
+                             a2 = *reinterpret_cast<const ulonglong2 *>(a + 8 * kLd),
+                             a3 = *reinterpret_cast<const ulonglong2 *>(a + 8 * kLd + 8);
+            const unsigned long long av[8] = {a0.x, a0.y, a1.x, a1.y, a2.x, a2.y, a3.x, a3.y};
+            uint32_t b[kDigits][2];
+            digit_frags(b, nx[q & 1][0][0], nx[q & 1][0][1], nx[q & 1][0][2], nx[q & 1][0][3]);
+            split_products(acc[0], av, b);
+            if (two) {
+                digit_frags(b, nx[q & 1][1][0], nx[q & 1][1][1], nx[q & 1][1][2], nx[q & 1][1][3]);
+                split_products(acc[1], av, b);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int r = g + 8 * (u >> 1), t = cb + 8 * h + t2 + (u & 1);
+                if (h == 0 || two) part[kw][r * kCols + t - col0] = split_value(acc[h], u) * chunk_scale(Er[r], Ex[t]);
+            }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int o = 0; o < kOut; ++o) {
+        const int e = threadIdx.x + 128 * o, r = e / kCols, t = col0 + e % kCols;
+        if (r0 + r >= M || t >= T) continue;
+        double v = 0.0;
+        if (!bad) {
+            v = part[0][e];
+#pragma unroll
+            for (int k = 1; k < KW; ++k) v += part[k][e];
+        } else {  // not finite, or beyond the doubles' range: plain FP64
+#pragma unroll 1
+            for (int k = 0; k < kc; ++k) v = fma(SrcF64::value(A.raw(r0 + r, k)), x[(int64_t)k * T + t], v);
+        }
+        C[(r0 + r) * T + t] = old[o] - v;
+    }
+}
+
+// KW by the number of blocks: as many warps along k as keep the blocks to four for each of the 152 SMs
+// (N = 10,242, T = 64: two 4.43 ms a step, four 4.20, eight 4.21).
+int launch_update(const SrcF64 &A, int64_t M, int kc, const double *x, int T, int Tp, const unsigned long long *D,
+                  const int *Ex, double *C, cudaStream_t s) {
+    const int64_t rows = (M + 15) / 16;
+    auto grid = [&](int kw) { return dim3((unsigned)rows, (unsigned)((T * kw + 63) / 64)); };
+    auto fits = [&](int kw) { return rows * ((T * kw + 63) / 64) <= kUpdateBlocks; };
+    if (fits(4) || T <= 16) launch_after_prologue(solve_update<4>, grid(4), 128, 0, s, A, M, kc, x, T, Tp, D, Ex, C);
+    else if (fits(2) || T <= 32) launch_after_prologue(solve_update<2>, grid(2), 128, 0, s, A, M, kc, x, T, Tp, D, Ex, C);
+    else launch_after_prologue(solve_update<1>, grid(1), 128, 0, s, A, M, kc, x, T, Tp, D, Ex, C);
+    return launch_status("solve_update");
 }
 
 __global__ void solve_gather(const double *__restrict__ Q, const int32_t *__restrict__ perm, int64_t N, int T,
@@ -431,7 +595,7 @@ int product(const Src &A, int64_t M, int64_t K, const V *x, int T, O *out, void 
     double *part = (double *)((char *)ws + p.digits + p.exps);
     RBFSL_CUDA_TRY(cudaMemsetAsync(Ex, 0, p.exps, s));
     x_digits<V><<<dim3((unsigned)nchunk, (unsigned)((Tp + 31) / 32)), 256, 0, s>>>(x, K, T, Tp, D, Ex);
-    const int rc = launch_gemm<Src, V, false>(A, M, K, x, T, Tp, D, Ex, p.splits,
+    const int rc = launch_gemm<Src, V>(A, M, K, x, T, Tp, D, Ex, p.splits,
                                               p.part ? part : reinterpret_cast<double *>(out), s);
     if (rc || !p.part) return rc;
     const int64_t cnt = M * T;
@@ -493,11 +657,11 @@ int split_solve(const double *LU, const int32_t *perm, int64_t N, const double *
         const int upper = j >= b;
         const int64_t r0 = (upper ? 2 * b - 1 - j : j) * kChunk, nb = std::min<int64_t>(kChunk, N - r0);
         int *ex = Ex + j * (Tp + 1);
-        solve_diag<<<(unsigned)Tp, 128, 0, s>>>(inv, off, N, r0, C, T, Tp, upper, D, ex);
+        launch_after_prologue(solve_diag, dim3((unsigned)Tp), 128, 0, s, inv, off, N, r0, C, T, Tp, upper, D, ex);
         const int64_t first = upper ? 0 : r0 + nb, rows = upper ? r0 : N - r0 - nb;
         if (rows <= 0) continue;
         const SrcF64 A{LU + first * N + r0, N};
-        const int rc = launch_gemm<SrcF64, double, true>(A, rows, nb, C + r0 * T, T, Tp, D, ex, 1, C + first * T, s);
+        const int rc = launch_update(A, rows, (int)nb, C + r0 * T, T, Tp, D, ex, C + first * T, s);
         if (rc) return rc;
     }
     return launch_status("global_solve");

@@ -12,6 +12,7 @@
 namespace rbfsl {
 
 constexpr int kDigits = 8, kGroups = 9;
+constexpr unsigned long long kZeroDigits = 0x8080808080808080ULL;  // digits_of(0, E)
 
 // Field of x's exponent (biased, 0 for zero and subnormals, 0x7ff for infinities and NaN).
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }

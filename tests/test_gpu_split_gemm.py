@@ -102,3 +102,23 @@ def test_solve_under_capture():
     g.replay()
     torch.cuda.synchronize()
     assert (c - ref).abs().max().item() <= 1e-9 * ref.abs().max().item()
+
+
+# the update's three arrangements (warps along the inner dimension 4, 2 and 1, by blocks of 16 rows) and their
+# edges: 16, 17, 32, 33 and 64 columns over 128 + 1 to 5,002 rows, against the solve column by column
+@pytest.mark.parametrize("N,T", [(129, 16), (1300, 17), (2700, 33), (2700, 64), (5002, 34), (5002, 64)])
+def test_solve_update_arrangements(N, T):
+    X = inputs.nodes(N, 6)
+    LU = torch.empty((N, N), dtype=torch.float64, device=DEV)
+    perm = torch.empty(N, dtype=torch.int32, device=DEV)
+    rbfsl.rbfsl_global_factor_chol(_t(X), rbfsl.IMQ, 0.1 * np.sqrt(N), LU, perm)
+    q = _t(np.random.default_rng(N + T).standard_normal((N, T)))
+    c, one = torch.empty_like(q), torch.empty((N, 1), dtype=torch.float64, device=DEV)
+    rbfsl.rbfsl_global_solve(LU, perm, q, c)
+    L = torch.tril(LU, -1) + torch.eye(N, dtype=torch.float64, device=DEV)
+    r = L @ (torch.triu(LU) @ c) - q[perm.long()]
+    for t in (0, T - 1):
+        rbfsl.rbfsl_global_solve(LU, perm, q[:, t:t + 1].contiguous(), one)
+        assert (c[:, t:t + 1] - one).abs().max() <= 1e-10 * one.abs().max()
+    A_inf = (L.abs() @ torch.triu(LU).abs()).sum(1).max().item()
+    assert r.abs().max().item() <= lu_residual_bound(N, A_inf, c.cpu().numpy())
