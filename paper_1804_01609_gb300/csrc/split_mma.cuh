@@ -117,7 +117,7 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo) {
     const unsigned long long L = (unsigned long long)l << 32, h = small ? L : (unsigned long long)hi;
     const int z = __clzll((long long)h) & 63;
     const unsigned long long m = (h << z) | (small || z == 0 ? 0 : L >> (64 - z));
-    const unsigned long long r = (m + (1u << 10)) >> 11;  // 53 bits, or 2^53
+    const unsigned long long r = (m >> 11) + ((m >> 10) & 1);  // 53 bits, or 2^53
     const unsigned long long bits = ((unsigned long long)(63 - z - (small ? 64 : 0) + 1022) << 52) + r;
     return __longlong_as_double((long long)(h == 0 ? 0 : bits | ((unsigned long long)neg << 63)));
 }
