@@ -303,7 +303,7 @@ __device__ __forceinline__ bool knn_warp(const KnnGrid &g, double qx, double qy,
     int bn = 0x7fffffff;
     for (int iter = 0; iter < 40; ++iter) {
         total = 0;
-        const double rb = sqrt(r2) * (1.0 + 1e-9) + 1e-15;
+        const float rb = sqrtf((float)r2);  // for the cells' tests, whose margins cover its rounding
         const long long r2b = __double_as_longlong(r2);
         grid_ball_foreach(g, qx, qy, qz, rb, lane, [&](int p, bool on) {
             double d2 = 0.0;

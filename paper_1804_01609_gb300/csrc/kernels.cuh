@@ -74,9 +74,9 @@ __device__ __forceinline__ int cell_coord(double v, double inv_cell, int G) {
 // the grid's border hold every point beyond it and are not narrowed on that side.
 template <typename F>
 __device__ __forceinline__ void grid_ball_foreach(const KnnGrid &g, double qx, double qy, double qz,
-                                                  double rb, int lane, F f) {
-    const float x = (float)qx, y = (float)qy, z = (float)qz, r = (float)rb * 1.00001f + 1e-6f;
-    const float inv = (float)g.inv_cell, edge = 1.0f / inv;
+                                                  float rb, int lane, F f) {
+    const float x = (float)qx, y = (float)qy, z = (float)qz, r = rb * 1.00001f + 1e-6f;
+    const float inv = 0.5f * (float)g.G, edge = 1.0f / inv;
     const int G = g.G;
     auto cell = [&](float v, float margin) {
         const int c = (int)floorf((v + 1.0f) * inv + margin);
@@ -123,9 +123,9 @@ __device__ __forceinline__ void grid_ball_foreach(const KnnGrid &g, double qx, d
 
 // The same for one thread: f(p) for the sorted positions p of the cells that the ball touches.
 template <typename F>
-__device__ __forceinline__ void grid_ball_rows(const KnnGrid &g, double qx, double qy, double qz, double rb, F f) {
-    const float x = (float)qx, y = (float)qy, z = (float)qz, r = (float)rb * 1.00001f + 1e-6f;
-    const float inv = (float)g.inv_cell, edge = 1.0f / inv;
+__device__ __forceinline__ void grid_ball_rows(const KnnGrid &g, double qx, double qy, double qz, float rb, F f) {
+    const float x = (float)qx, y = (float)qy, z = (float)qz, r = rb * 1.00001f + 1e-6f;
+    const float inv = 0.5f * (float)g.G, edge = 1.0f / inv;
     const int G = g.G;
     auto cell = [&](float v, float margin) {
         const int c = (int)floorf((v + 1.0f) * inv + margin);

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(128) pu_members_kernel(KnnGrid g, const double
     const double ox = Om[3 * l], oy = Om[3 * l + 1], oz = Om[3 * l + 2];
     if (lane == 0) cnt[warp] = 0;
     __syncwarp();
-    grid_ball_foreach(g, ox, oy, oz, R * (1.0 + 1e-9) + 1e-15, lane, [&](int p, bool on) {
+    grid_ball_foreach(g, ox, oy, oz, (float)R, lane, [&](int p, bool on) {
         if (on && sqrt(sqdist_rn(ox, oy, oz, g.sx[p], g.sy[p], g.sz[p])) < R) {
             const int slot = atomicAdd(&cnt[warp], 1);
             if (slot < kPuMaxCand) buf[warp][slot] = g.sid[p];
@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(64) pu_points_kernel(KnnGrid cg, double Rr, in
     // patches with |p - omega_l| < R: distances squared, the root only where rounding could decide
     const double hi = Rr * Rr * (1.0 + 1e-15), lo = Rr * Rr * (1.0 - 1e-15);
     int n = 0;
-    grid_ball_rows(cg, px, py, pz, Rr * (1.0 + 1e-9) + 1e-15, [&](int c) {
+    grid_ball_rows(cg, px, py, pz, (float)Rr, [&](int c) {
         const double d2 = sqdist_rn(px, py, pz, cg.sx[c], cg.sy[c], cg.sz[c]);
         if (!(d2 < hi) || (d2 > lo && !(sqrt(d2) < Rr))) return;
         if (n < kPuMaxPatches) {
