@@ -275,7 +275,7 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
         const int i = tri_row(e) + 1, j = e - tri(i - 1);
         const double dx = cx[i] - cx[j], dy = cy[i] - cy[j], dz = cz[i] - cz[j];
         const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        if (d2 == 0.0 && i < n) st[0] = RBFSL_ESINGULAR;  // two coincident nodes: two equal rows
+        if (__double_as_longlong(d2) == 0 && i < n) st[0] = RBFSL_ESINGULAR;  // two coincident nodes: two equal rows
         const double v = phs_pow(d2, half);
         if (i < M) {
             A11[tri(i - 1) + j] = v;
@@ -585,7 +585,9 @@ __host__ __device__ inline int center_lanes(int n, int M) { return M <= 16 && n 
 
 // S: the stencil (n), F: its factors, order: pivot order; l: lane within the point's group. The
 // other groups of the warp run the same steps. Returns the weights (shared, stencil order).
-template <int kLanes>
+// kOwnY: whether the group evaluates the harmonics itself; else the caller has left them at
+// sm + M * M + n, a barrier before the call.
+template <int kLanes, bool kOwnY = true>
 __device__ __forceinline__ double *center_point_reduced(const double *__restrict__ X, const int32_t *__restrict__ S,
                                                         const double *__restrict__ F,
                                                         const int32_t *__restrict__ order, int n, int M, int ell,
@@ -600,7 +602,7 @@ __device__ __forceinline__ double *center_point_reduced(const double *__restrict
         const double dx = px - X[3 * s], dy = py - X[3 * s + 1], dz = pz - X[3 * s + 2];
         phi[j] = phs_pow(fma(dz, dz, fma(dy, dy, dx * dx)), half);
     }
-    sh_eval_lanes(ell, px, py, pz, l, [&](int c, double v) { y[c] = v; });
+    if (kOwnY) sh_eval_lanes(ell, px, py, pz, l, [&](int c, double v) { y[c] = v; });
     __syncwarp();
     for (int k = 0; k < M; ++k) {  // y R^-1
         const double yk = y[k];

@@ -162,13 +162,23 @@ __global__ void __launch_bounds__(128) center_reduced_kernel(
     const double *__restrict__ P, int32_t *__restrict__ I, WT *__restrict__ W, int32_t *__restrict__ status) {
     extern __shared__ double sm[];
     const int grp = threadIdx.x / kLanes, l = threadIdx.x % kLanes;
-    const int64_t i0 = (int64_t)blockIdx.x * (128 / kLanes) + grp;
+    constexpr int kPoints = 128 / kLanes;
+    const int64_t b0 = (int64_t)blockIdx.x * kPoints, i0 = b0 + grp;
+    // the harmonics of the block's points, a thread per point and order: on the FP64 pipe a warp
+    // instruction costs the same whatever its active lanes
+    for (int f = threadIdx.x; f < kPoints * (ell + 1); f += 128) {
+        const int p = f / (ell + 1);
+        const int64_t i = b0 + p < Nq ? b0 + p : Nq - 1;
+        double *y = sm + (size_t)p * center_reduced_doubles(n, M) + M * M + n;
+        sh_eval_lanes(ell, P[3 * i], P[3 * i + 1], P[3 * i + 2], f - p * (ell + 1), [&](int c, double v) { y[c] = v; });
+    }
+    __syncthreads();
     if (i0 - grp % (32 / kLanes) >= Nq) return;  // the whole warp past the end
     const bool on = i0 < Nq;                     // a group past the end repeats the last point
     const int64_t i = on ? i0 : Nq - 1;
     const int64_t kc = Kc[i], k = kc < 0 ? 0 : kc;
     const int32_t *S = Ik + k * n;
-    double *w = center_point_reduced<kLanes>(X, S, F + (size_t)k * CenterLayout(n, M).total, order + (size_t)k * n, n, M,
+    double *w = center_point_reduced<kLanes, false>(X, S, F + (size_t)k * CenterLayout(n, M).total, order + (size_t)k * n, n, M,
                                              ell, half, P[3 * i], P[3 * i + 1], P[3 * i + 2],
                                              sm + (size_t)grp * center_reduced_doubles(n, M), l);
     if (!on) return;
