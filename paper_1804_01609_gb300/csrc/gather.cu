@@ -55,9 +55,10 @@ __global__ void __launch_bounds__(256) gather_dot_kernel(const int32_t *__restri
     }
 }
 
-// Vectorised variant for T a multiple of the vector width V (4 floats or 2 doubles = 16 B):
-// a row group of G = T / V lanes serves one row (32 / G rows per warp), every lane owning V
-// consecutive tracers, so each gathered q row is read as G 16-byte pieces. Members are taken in
+// Rows of at most 32 pieces of V values (V = 4 floats or 2 doubles = 16 B where T is a multiple of it,
+// else V = 1): a row group of G = T / V lanes serves one row (32 / G rows per warp), every lane owning V
+// consecutive tracers, so each gathered q row is read as G pieces. (N = 2,562, n = 31, one FP64 tracer, a
+// lane per row: 22 us by the scalar kernel, one gather in flight per lane; now 8.4.) Members are taken in
 // batches of kGatherBatch: the batch's indices and weights are loaded first (the G lanes of a
 // row group read the same words), then all its q pieces are requested before the first is
 // used, so a lane keeps kGatherBatch gathers in flight instead of one; with 16-byte aligned rows
@@ -111,9 +112,10 @@ __global__ void __launch_bounds__(256, 4) gather_dot_vec_kernel(const int32_t *_
                 sb[b] = iv.x; sb[b + 1] = iv.y; sb[b + 2] = iv.z; sb[b + 3] = iv.w;
             }
             constexpr int WV = 16 / (int)sizeof(R);
+            using WVec = typename std::conditional<sizeof(R) == 8, double2, float4>::type;
 #pragma unroll
             for (int b = 0; b < kGatherBatch; b += WV) {
-                const RV wv = *reinterpret_cast<const RV *>(Wr + j0 + b);
+                const WVec wv = *reinterpret_cast<const WVec *>(Wr + j0 + b);
                 const R *wr = reinterpret_cast<const R *>(&wv);
 #pragma unroll
                 for (int u = 0; u < WV; ++u) wb[b + u] = wr[u];
@@ -228,8 +230,8 @@ int launch_gather(const int32_t *idx, const void *w, int64_t Nq, int n, const vo
         int G = 1;
         while (G < need && G < 32) G <<= 1;
         const int rows_per_warp = kWarp / G;
-        const int threads = 256;
         const int64_t warps = (Nq + rows_per_warp - 1) / rows_per_warp;
+        const int threads = warps < 152 * 16 ? 64 : 256;  // few warps: spread over the SMs
         const unsigned blocks = (unsigned)((warps * kWarp + threads - 1) / threads);
         const bool vl = n % 4 == 0 && (uintptr_t)idx % 16 == 0 && (uintptr_t)w % 16 == 0;
         auto go = [&](auto k) {
@@ -241,31 +243,34 @@ int launch_gather(const int32_t *idx, const void *w, int64_t Nq, int n, const vo
         else go(gather_dot_pair_kernel<1, false>);
         return launch_status("gather_dot_pair");
     }
-    const int V = dtype == RBFSL_F64 ? 2 : 4;
+    // FP64 and FP32: 16 bytes of a row per lane where the rows are aligned for it, else one value; rows of
+    // up to 32 lanes' pieces
     const bool aligned = ((uintptr_t)q % 16 == 0) && ((uintptr_t)q_out % 16 == 0);
-    if (T % V == 0 && T / V <= 32 && aligned) {
-        int G = 1;
-        while (G < T / V) G <<= 1;  // a power of two >= T / V lanes per row
-        if (G == T / V) {
-            const int rows_per_warp = kWarp / G;
-            const int threads = 256;
-            const int64_t warps = (Nq + rows_per_warp - 1) / rows_per_warp;
-            const unsigned blocks = (unsigned)((warps * kWarp + threads - 1) / threads);
-            const bool vl = n % 4 == 0 && (uintptr_t)idx % 16 == 0 && (uintptr_t)w % 16 == 0;
-            if (dtype == RBFSL_F64 && vl)
-                gather_dot_vec_kernel<double, double2, 2, false, true><<<blocks, threads, 0, s>>>(
-                    idx, (const double *)w, Nq, n, (const double *)q, T, G, (double *)q_out);
-            else if (dtype == RBFSL_F64)
-                gather_dot_vec_kernel<double, double2, 2, false, false><<<blocks, threads, 0, s>>>(
-                    idx, (const double *)w, Nq, n, (const double *)q, T, G, (double *)q_out);
-            else if (vl)
-                gather_dot_vec_kernel<float, float4, 4, true, true><<<blocks, threads, 0, s>>>(
-                    idx, (const float *)w, Nq, n, (const float *)q, T, G, (float *)q_out);
-            else
-                gather_dot_vec_kernel<float, float4, 4, true, false><<<blocks, threads, 0, s>>>(
-                    idx, (const float *)w, Nq, n, (const float *)q, T, G, (float *)q_out);
-            return launch_status("gather_dot_vec");
+    const int full = dtype == RBFSL_F64 ? 2 : 4, V = T % full == 0 && aligned ? full : 1, G = T / V;
+    if (G <= 32) {
+        const int rows_per_warp = kWarp / G;
+        const int64_t warps = (Nq + rows_per_warp - 1) / rows_per_warp;
+        const int threads = warps < 152 * 16 ? 64 : 256;  // few warps: spread over the SMs
+        const unsigned blocks = (unsigned)((warps * kWarp + threads - 1) / threads);
+        const bool vl = n % 4 == 0 && (uintptr_t)idx % 16 == 0 && (uintptr_t)w % 16 == 0;
+        auto go = [&](auto k, auto *t) {
+            using R = typename std::remove_pointer<decltype(t)>::type;
+            k<<<blocks, threads, 0, s>>>(idx, (const R *)w, Nq, n, (const R *)q, T, G, (R *)q_out);
+        };
+        if (dtype == RBFSL_F64) {
+            double *t = nullptr;
+            if (V == 2 && vl) go(gather_dot_vec_kernel<double, double2, 2, false, true>, t);
+            else if (V == 2) go(gather_dot_vec_kernel<double, double2, 2, false, false>, t);
+            else if (vl) go(gather_dot_vec_kernel<double, double, 1, false, true>, t);
+            else go(gather_dot_vec_kernel<double, double, 1, false, false>, t);
+        } else {
+            float *t = nullptr;
+            if (V == 4 && vl) go(gather_dot_vec_kernel<float, float4, 4, true, true>, t);
+            else if (V == 4) go(gather_dot_vec_kernel<float, float4, 4, true, false>, t);
+            else if (vl) go(gather_dot_vec_kernel<float, float, 1, true, true>, t);
+            else go(gather_dot_vec_kernel<float, float, 1, true, false>, t);
         }
+        return launch_status("gather_dot_vec");
     }
     int L = 1;
     while (L < T && L < 32) L <<= 1;
