@@ -14,7 +14,7 @@
 //                             reset.
 // The per-point arithmetic is the same device code as the single-problem kernels
 // (device_ops.cuh), so a problem's result is bit-identical alone or in any batch.
-// Tile shape per (n, ell) class: one warp per point (four points per 128-thread block) or four
+// Tile shape per (n, ell) class: one warp per point (four points per 128-thread block), two or four
 // warps per point; chosen by rbfsl_batch_autotune (timed) or by a size rule.
 #include <algorithm>
 #include <cmath>
@@ -118,6 +118,35 @@ __device__ __forceinline__ void batch_gather(const BatchDesc &b, const double *w
     }
 }
 
+// One point of a direct-mode problem by NW warps (thread t of the group) in the region A.
+template <int NW>
+__device__ __forceinline__ void batch_direct_point(const BatchDesc &b, double *A, int64_t i, int n, int m, int cap,
+                                                   int t) {
+    const int warp = t >> 5, lane = t & 31;
+    int32_t *S = reinterpret_cast<int32_t *>(A + weights_doubles(n, m, b.ell, b.half));
+    double *bd = A;  // aliases the region (see batch_point_doubles)
+    int *bi = reinterpret_cast<int *>(bd + cap);
+    const double px = b.xi[3 * i], py = b.xi[3 * i + 1], pz = b.xi[3 * i + 2];
+    if (warp == 0) {
+        const bool ok = knn_warp(b.grid, px, py, pz, n, cap, bd, bi, lane);
+        for (int j = lane; j < n; j += 32) S[j] = ok ? bi[j] : -1;
+    }
+    group_sync<NW>();
+    double *wv = nullptr;
+    const int rc = weights_point<NW>(A, b.X, S, n, m, b.ell, b.half, px, py, pz, t, wv);
+    if (warp != 0) return;
+    if (rc == RBFSL_OK) {
+        batch_gather(b, wv, S, i, lane);
+    } else {
+        const int in = (int)(b.step & 1);
+        for (int c = lane; c < b.T; c += 32) {
+            if (b.mixed) ((float2 *)b.q[in ^ 1])[i * b.T + c] = make_float2(NAN, NAN);
+            else ((double *)b.q[in ^ 1])[i * b.T + c] = NAN;
+        }
+    }
+    if (lane == 0) b.status[i] = rc;
+}
+
 // Tiles [tile_begin, tile_end) of the table's problems [p_begin, p_begin + np) (one class).
 __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__restrict__ d, int p_begin, int np,
                                                           int64_t tile_begin, int64_t tile_end,
@@ -140,7 +169,7 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
         if (b.ppt == 4 || b.mode == RBFSL_CENTER) {
             // one warp per point
             const int64_t i = (tile - b.tile0) * 4 + warp;
-            if (i >= b.N) continue;
+            if (i >= b.N) continue;  // (ends at the next tile's barriers)
             double *base = sm + (size_t)warp * per;
             double *A = base;
             int32_t *S = reinterpret_cast<int32_t *>(base + weights_doubles(n, m, b.ell, b.half));  // direct only
@@ -178,34 +207,11 @@ __global__ void __launch_bounds__(128, 4) batch_solve_kernel(const BatchDesc *__
                 }
             }
             if (lane == 0) b.status[i] = rc;
+        } else if (b.ppt == 2) {
+            const int64_t i = (tile - b.tile0) * 2 + (t >> 6);
+            if (i < b.N) batch_direct_point<2>(b, sm + (size_t)(t >> 6) * per, i, n, m, cap, t & 63);
         } else {
-            // four warps per point (direct mode)
-            const int64_t i = tile - b.tile0;
-            double *A = sm;
-            int32_t *S = reinterpret_cast<int32_t *>(sm + weights_doubles(n, m, b.ell, b.half));
-            double *bd = sm;  // aliases the region (see batch_point_doubles)
-            int *bi = reinterpret_cast<int *>(bd + cap);
-            const double px = b.xi[3 * i], py = b.xi[3 * i + 1], pz = b.xi[3 * i + 2];
-            if (warp == 0) {
-                const bool ok = knn_warp(b.grid, px, py, pz, k, cap, bd, bi, lane);
-                for (int j = lane; j < n; j += 32) S[j] = ok ? bi[j] : -1;
-            }
-            __syncthreads();
-            double *wv = nullptr;
-            const int rc = weights_point<4>(A, b.X, S, n, m, b.ell, b.half, px, py, pz, t, wv);
-            if (warp == 0) {
-                if (rc == RBFSL_OK) {
-                    batch_gather(b, wv, S, i, lane);
-                } else {
-                    const int in = (int)(b.step & 1);
-                    for (int c = lane; c < b.T; c += 32) {
-                        if (b.mixed) ((float2 *)b.q[in ^ 1])[i * b.T + c] = make_float2(NAN, NAN);
-                        else ((double *)b.q[in ^ 1])[i * b.T + c] = NAN;
-                    }
-                }
-                if (lane == 0) b.status[i] = rc;
-            }
-            __syncthreads();
+            batch_direct_point<4>(b, sm, tile - b.tile0, n, m, cap, t);
         }
     }
 }
@@ -287,7 +293,8 @@ int default_ppt(const rbfsl_batch *b, int n, int ell, int mode) {
     auto it = b->tile_rule.find(class_key(n, ell));
     if (it != b->tile_rule.end()) return it->second;
     const int m = n + (ell + 1) * (ell + 1);
-    return weights_doubles(n, m, ell, 0) * 8 > kWeightsSmallBytes || reduced_on_tensor(m - n) ? 1 : 4;  // the single-problem rule
+    const int bytes = weights_doubles(n, m, ell, 0) * 8;  // the single-problem rule
+    return bytes <= kWeightsSmallBytes && !reduced_on_tensor(m - n) ? 4 : bytes <= kWeightsPairBytes ? 2 : 1;
 }
 
 void free_problem(HostProblem &h) {
@@ -330,10 +337,10 @@ int rebuild(rbfsl_batch *b) {
             d.node0 = nodes;
             d.tile0 = tiles;
             nodes += d.N;
-            tiles += d.ppt == 4 ? (d.N + 3) / 4 : d.N;
+            tiles += (d.N + d.ppt - 1) / d.ppt;
             const int cap = knn_cap(d.mode == RBFSL_DIRECT ? d.n : 1);
             const int per = batch_point_doubles(d.mode, d.n, d.m, d.ell, d.half, cap) * 8;
-            cl.smem = std::max(cl.smem, d.ppt == 4 ? 4 * per : per);
+            cl.smem = std::max(cl.smem, d.ppt * per);
             b->slot_of[id] = (int)tab.size();
             tab.push_back(d);
         }
@@ -648,7 +655,7 @@ int rbfsl_batch_set_graph(rbfsl_batch *b, int use_graph) {
 }
 
 // Time the persistent solve kernel for each direct-mode (n, ell) class of the batch with one
-// warp per point and with four warps per point, keep the faster. The timing launches run on
+// warp, two and four warps per point, keep the fastest. The timing launches run on
 // the current departure points and leave the fields, times and step counters unchanged.
 int rbfsl_batch_autotune(rbfsl_batch *b, int *choices, int max_choices) {
     RBFSL_CHECK_ARG(b != nullptr, "batch_autotune: null batch");
@@ -672,8 +679,8 @@ int rbfsl_batch_autotune(rbfsl_batch *b, int *choices, int max_choices) {
         int best = 1;
         const int kn = (int)(key / 64), kell = (int)(key % 64), km = kn + (kell + 1) * (kell + 1);
         const int per_bytes = batch_point_doubles(RBFSL_DIRECT, kn, km, kell, 0, knn_cap(kn)) * 8;
-        for (int ppt : {4, 1}) {
-            if (ppt == 4 && 4 * per_bytes > max_smem) continue;
+        for (int ppt : {4, 2, 1}) {
+            if (ppt > 1 && ppt * per_bytes > max_smem) continue;
             // only this class active, with the candidate tile shape
             std::vector<int> saved;
             for (auto &h : b->probs) {

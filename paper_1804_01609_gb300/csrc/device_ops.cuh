@@ -403,6 +403,8 @@ __host__ __device__ inline int ldl_doubles(int n, int m) {
 }
 // Shared-memory bytes of one point up to which one warp takes a point (m <~ 45).
 constexpr int kWeightsSmallBytes = 12 * 1024;
+// ... up to which two warps take a larger point (eight points per SM).
+constexpr int kWeightsPairBytes = 28 * 1024;
 
 __device__ __forceinline__ int tri(int i) { return i * (i + 1) / 2; }
 
@@ -477,6 +479,20 @@ __device__ __forceinline__ double recip_nr(double d) {
     return fma(r, fma(-d, r, 1.0), r);
 }
 
+// Barrier of a point's group of NW warps: a warp, a 64-thread half of the block (two groups of two warps
+// may run apart), or the block.
+template <int NW>
+__device__ __forceinline__ void group_sync() {
+    if (NW == 1) {
+        __syncwarp();
+    } else if (NW == 2) {  // fixed numbers: a computed one reserves all sixteen of the block's barriers
+        if (threadIdx.x < 64) asm volatile("bar.sync 1, 64;" ::: "memory");
+        else asm volatile("bar.sync 2, 64;" ::: "memory");
+    } else {
+        __syncthreads();
+    }
+}
+
 // Weights of one point by a group of NW warps (thread t of the group). Assembles the packed
 // lower triangle of A~ and b (Eqs. rbf_poly, rbf_poly_linsys), factorises with Bunch-Kaufman
 // pivoting (alpha = (1 + sqrt 17) / 8; column maximum lambda at row r (smaller row on a tie),
@@ -511,7 +527,7 @@ __device__ __forceinline__ int weights_point_ldl(double *__restrict__ R, const d
     int *perm = reinterpret_cast<int *>(slot + 16), *ptype = perm + m, *st = ptype + m;
     // st[0]: error flag, st[1]: pivot size of the current step, st[2]: close the panel first
     auto gsync = [] {
-        if (NW == 1) __syncwarp(); else __syncthreads();
+        group_sync<NW>();
     };
     out = cx;
     if (t == 0) st[0] = 0;

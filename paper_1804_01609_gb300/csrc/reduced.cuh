@@ -159,7 +159,7 @@ __device__ __forceinline__ int weights_point_reduced(double *__restrict__ R, con
     int *st = reinterpret_cast<int *>(R + lay.ints), *ord = st + 6;
     // st[0]: error code, st[1]: breakdown, st[2..4]: largest exponent fields of W, A11 and Y
     auto gsync = [] {
-        if (NW == 1) __syncwarp(); else __syncthreads();
+        group_sync<NW>();
     };
     out = cx;
     if (t < 5) st[t] = 0;
@@ -558,7 +558,7 @@ __device__ __forceinline__ int weights_point(double *__restrict__ R, const doubl
                            ? weights_point_reduced<NW, kTensor>(R, X, stencil, n, M, ell, half, px, py, pz, t, out)
                            : weights_point_reduced<NW, false>(R, X, stencil, n, M, ell, half, px, py, pz, t, out);
         if (rc <= 0) return rc;
-        if (NW == 1) __syncwarp(); else __syncthreads();  // every thread has read the breakdown flag
+        group_sync<NW>();  // every thread has read the breakdown flag
     }
     return weights_point_ldl<NW>(R, X, stencil, n, m, ell, half, px, py, pz, t, out);
 }

@@ -65,14 +65,13 @@ struct WeightsArgs {
     int32_t *status;
 };
 
-// NW warps per point (1 or 4). With NW = 1 a block holds blockDim/32 independent points and
+// NW warps per point (1, 2 or 4). With NW = 1 a block holds blockDim/32 independent points and
 // the group barrier is __syncwarp; with NW > 1 a block is one point and uses __syncthreads. kBlocks:
 // the blocks per SM that the registers are bounded for: seven for one warp per point (72 registers);
-// with four warps, whose digit products want 117, four where shared memory allows no more (m = 109)
-// and five (96 registers, 40 bytes spilled) where it does (m = 71: 6.6 ms against 7.1 ms at
-// N = 40,962; m = 109 16.9 against 16.4).
+// with two and four warps, whose digit products want 117 to 128, what shared memory allows (eight points of
+// two warps, five or four of four).
 template <int NW, int kBlocks, typename WT>
-__global__ void __launch_bounds__(128, kBlocks) weights_kernel(WeightsArgs a, WT *__restrict__ W) {
+__global__ void __launch_bounds__(NW == 2 ? 64 : 128, kBlocks) weights_kernel(WeightsArgs a, WT *__restrict__ W) {
     extern __shared__ double smem[];
     constexpr int GT = NW * kWarp;
     const int g = threadIdx.x / GT, t = threadIdx.x % GT;
@@ -120,8 +119,11 @@ int launch_weights(const double *x, const int32_t *idx, int64_t Nq, int n, int e
     a.region_doubles = weights_doubles(n, a.m, ell, a.half);
     const int bytes = a.region_doubles * 8;
     if (bytes > kWeightsSmallBytes || (reduced_form(n, ell, a.half) && reduced_on_tensor(a.m - n))) {
-        // larger systems (m >~ 45, or with the products on the tensor cores): four warps per point
-        // (one per SM sub-partition), one point per block; five blocks need 1/5 of 227 KB each
+        // larger systems (m >~ 45, or with the products on the tensor cores), one point per block: two warps
+        // per point while eight points fit an SM's 227 KB (more points overlap each other's serial steps:
+        // m = 71 at N = 12,347 1.73 ms, four warps and five points 1.90), else four warps; five blocks need
+        // 1/5 of it each
+        if (bytes <= kWeightsPairBytes) return launch_weights_typed<2, 8>(a, 1, w, w_dtype, s);
         return bytes <= 44 * 1024 ? launch_weights_typed<4, 5>(a, 1, w, w_dtype, s)
                                   : launch_weights_typed<4, 4>(a, 1, w, w_dtype, s);
     }

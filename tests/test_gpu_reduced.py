@@ -109,3 +109,29 @@ def test_centre_stencils_on_coarse_nodes(orc, N, n, ell, p):
     err = np.abs(c.get_q() - ref).max()
     c.close()
     assert err <= 5 * floor + 1e-12 * np.abs(q).max()
+
+
+# two warps per point (up to 28 KB a point): in the batch two points share a block, the last block of an odd
+# node count holds one; the context's kernel has a block per point
+@pytest.mark.parametrize("n,ell,N", [(33, 3, 901), (55, 3, 643), (60, 3, 1200)])
+def test_two_warps_per_point_in_a_batch(n, ell, N):
+    X = inputs.nodes(N, 3)
+    q = np.stack([inputs.gaussian_hills(X, [[0.6, 0.0, 0.8]]), inputs.cosine_bell(X, [1.0, 0.0, 0.0], 0.9)], axis=1)
+    vp = inputs.deformation_params(2.0, 1.0)
+    b = rbfsl.Batch(0, stream=torch.cuda.Stream())
+    i = b.add(X, q, n, ell, 2 * ell + 1, rbfsl.VEL_DEFORM_Y2, vp, 1.0 / 60, mode=rbfsl.DIRECT, precision=rbfsl.FP64)
+    b.step(2)
+    got = b.get_q(i)
+    b.close()
+    c = rbfsl.Context(0)
+    c.set_nodes(X)
+    c.set_velocity(rbfsl.VEL_DEFORM_Y2, vp)
+    c.set_method(rbfsl.LOCAL, rbfsl.DIRECT)
+    c.set_stencil_size(n)
+    c.set_sh_degree(ell)
+    c.set_kernel(rbfsl.PHS, 2 * ell + 1)
+    c.set_dt(1.0 / 60)
+    c.set_tracers(q)
+    c.step(2)
+    np.testing.assert_array_equal(got, c.get_q())
+    c.close()
