@@ -50,12 +50,11 @@ struct KnnGrid {
     const double *sx, *sy, *sz;
     const int32_t *sid, *cell_start;
     int G;
-    double inv_cell;
     double r2_per_k;
 };
 
 inline KnnGrid grid_view(const rbfsl_knn_index *ix) {
-    return KnnGrid{ix->sx, ix->sy, ix->sz, ix->sid, ix->cell_start, ix->G, ix->G / 2.0, ix->r2_per_k};
+    return KnnGrid{ix->sx, ix->sy, ix->sz, ix->sid, ix->cell_start, ix->G, ix->r2_per_k};
 }
 
 __device__ __forceinline__ int cell_coord(double v, double inv_cell, int G) {

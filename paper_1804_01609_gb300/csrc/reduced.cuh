@@ -23,7 +23,7 @@
 // whole system (device_ops.cuh) 30.3 ms (FP64 pipe 80% busy); reduced form with FP64 products
 // 24.4 ms, 9,817 FP64 warp instructions per point (85% busy); products on the tensor cores 18.5 ms,
 // 6,138 (72%); panels of four columns instead of eight, digits formed once, split rows of W, the
-// search ahead and the FP32 first iterations 15.7 ms.
+// search ahead and the FP32 first iterations 15.7 ms, the digit sums made doubles by integers 15.0 ms.
 #pragma once
 
 #include "common.cuh"
@@ -573,7 +573,7 @@ __device__ __forceinline__ int weights_point(double *__restrict__ R, const doubl
 //
 // Bound: the FP64 pipe (two thirds of the multiplications of substituting through an LU factor of
 // the whole system, and a serial chain of 2 M steps instead of 2 (n + M)), then HBM (8 (n^2 + K (M + 1))
-// bytes per point). N = 40,962, n = 84 1.15 ms against 2.33 ms, N = 163,842, n = 31 0.90 ms against
+// bytes per point). N = 40,962, n = 84 0.97 ms against 2.33 ms, N = 163,842, n = 31 0.80 ms against
 // 1.91 ms for the LU factors, which stay for the systems without the reduced form.
 
 // Shared doubles of one point: P1's factor, phi (later z = D^-1 L^-1 g), Y(p), u, g (later w2) and the weights.

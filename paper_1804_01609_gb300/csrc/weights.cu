@@ -8,9 +8,9 @@
 // (reduced.cuh) or, for exponents above the harmonics' order and n <= M, as a whole by a blocked
 // Bunch-Kaufman L D L^T (weights_point_ldl): ~m^3 / 3 flops per point either way (m = n + M), bound
 // by GB300's FP64 rate. Small systems take one warp per point (four points per block); larger ones
-// four warps per point, several points per SM so that one point's serial steps overlap the others'
-// products. N = 40,962, reduced form against the indefinite factorisation: m = 109 15.7 ms against
-// 30.3 ms, m = 71 6.6 ms against 10.1 ms, m = 40 2.1 ms against 2.9 ms.
+// two or four warps per point, several points per SM so that one point's serial steps overlap the others'
+// products. N = 40,962, reduced form against the indefinite factorisation: m = 109 15.0 ms against
+// 30.3 ms, m = 71 (before two warps per point) 6.6 ms against 10.1 ms, m = 40 2.1 ms against 2.9 ms.
 #include <vector>
 
 #include "common.cuh"
