@@ -268,6 +268,12 @@ int launch_gemm(const Src &A, int64_t M, int64_t K, const V *x, int T, int Tp, c
 
 // ---- triangular solves with diagonal blocks of 128 rows
 constexpr int kB = 64;  // inverted triangular blocks (two to a diagonal block)
+// Condition of a block above which its inverse's product is corrected (solve_diag). Below it the product's
+// residual, relative to |T| |x|, is within four times substitution's (blocks of Gaussian and IMQ factors, N = 1,000 to
+// 4,999; from 64 on up to a hundred times); a correction of every block made the step of N = 4,999, T = 9
+// 2.21 instead of 1.89 ms and that of N = 10,242, T = 64 4.67 instead of 3.94, though nine tenths of their
+// blocks lie below 16.
+constexpr double kSolveCond = 16.0;
 
 // Programmatic dependent launch: the next kernel of the stream may start (its prologue runs beside this
 // kernel), and wait until every kernel before this one is complete. What an earlier kernel of the chain
@@ -295,10 +301,12 @@ void launch_after_prologue(void (*kernel)(P...), dim3 grid, int threads, int sme
 // Inverses of the 64 x 64 diagonal blocks of the unit lower (blockIdx.y = 0) and the upper factor
 // (1), column-major, and the 64 x 64 block that couples a diagonal block's halves (also
 // column-major): what the block substitution needs, laid out for its lanes. A block's inverse
-// replaces 64 dependent steps by a product. Rows and columns beyond N: the identity.
+// replaces 64 dependent steps by a product. Rows and columns beyond N: the identity. cond: the blocks'
+// Skeel condition numbers.
 __global__ void __launch_bounds__(64) solve_prepare(const double *__restrict__ LU, int64_t N, double *__restrict__ inv,
-                                                    double *__restrict__ off) {
+                                                    double *__restrict__ off, double *__restrict__ cond) {
     extern __shared__ double sm[];
+    __shared__ double z[kB];
     double *F = sm, *V = sm + kB * (kB + 1);  // the block (row-major) and its inverse (column-major), padded
     const int64_t j = blockIdx.x, r0 = j * kB;
     const int c = threadIdx.x, upper = blockIdx.y;
@@ -334,6 +342,21 @@ __global__ void __launch_bounds__(64) solve_prepare(const double *__restrict__ L
     __syncthreads();
     double *o = inv + (2 * j + upper) * kB * kB;
     for (int q = 0; q < kB; ++q) o[q * kB + c] = V[q * (kB + 1) + c];
+    {  // cond(T) = the largest row sum of |T^-1| |T|; a value that is not finite counts as large
+        double a = upper ? 0.0 : 1.0;
+        for (int q = upper ? c : 0; q < (upper ? kB : c); ++q) a += fabs(F[c * (kB + 1) + q]);
+        z[c] = a;
+        __syncthreads();
+        a = 0.0;
+        for (int q = 0; q < kB; ++q) a = fma(fabs(V[q * (kB + 1) + c]), z[q], a);
+        __syncthreads();
+        z[c] = a;
+        __syncthreads();
+        if (c == 0) {
+            for (int q = 1; q < kB; ++q) a = z[q] <= a ? a : z[q];
+            cond[2 * j + upper] = a <= 1e300 ? a : 1e300;
+        }
+    }
     if (upper ? !(j & 1) : (j & 1)) {  // lower: rows of an odd block, columns before it; upper: the other half
         const int64_t cb = upper ? r0 + kB : r0 - kB;
         double *p = off + (2 * (j >> 1) + upper) * kB * kB;
@@ -345,65 +368,104 @@ __global__ void __launch_bounds__(64) solve_prepare(const double *__restrict__ L
 }
 
 // One diagonal block (128 rows from r0) for one right-hand side per thread block: forward x1 =
-// L11^-1 y1, x2 = L22^-1 (y2 - L21 x1), backward the other way round; x replaces y and its digits go
-// to the update. Two threads to a row, each half of the columns. Bound: latency; a thread's 96 matrix
-// entries are loaded beside the kernel before (the columns of the padding, and those of a missing second
-// half, are the identity's).
-__global__ void __launch_bounds__(128) solve_diag(const double *__restrict__ inv, const double *__restrict__ off,
-                                                  int64_t N, int64_t r0, double *Y, int T, int Tp, int upper,
-                                                  unsigned long long *D, int *Ex) {
-    __shared__ double y[2 * kB], part[2 * kB];
+// T11^-1 y1, x2 = T22^-1 (y2 - T21 x1), backward the other way round; x replaces y and its digits go
+// to the update. A product with a 64 x 64 inverse alone is not backward stable: its residual grows with
+// the block's condition, and the blocks of flat kernels are badly conditioned (Gaussian, eps = 3 on 2,562
+// nodes: residual 1.8e-9 against substitution's 5e-11). Where cond(T) exceeds kSolveCond the product is
+// corrected once, x += T^-1 (y - T x), with the factor's own block T, which brings the residual back to
+// substitution's.
+// Eight warps: 16 rows and every second pair of columns each, a lane every fourth column; a triangle's empty
+// 16 x 16 tiles are left out, with the rows dealt so that the SM's four schedulers have equal work. Bound:
+// the FP64 pipe (a warp instruction keeps its scheduler's quarter busy for 64 cycles, which also hides the
+// one chain of FMAs a lane has) and latency; a thread's matrix entries are loaded beside the kernel before
+// (columns of the padding are the identity's in the inverses and zero in T, where x is zero too).
+__global__ void __launch_bounds__(256, 1) solve_diag(const double *__restrict__ LU, const double *__restrict__ inv,
+                                                     const double *__restrict__ off, const double *__restrict__ cond,
+                                                     int64_t N, int64_t r0, double *Y, int T, int Tp, int upper,
+                                                     unsigned long long *D, int *Ex) {
+    __shared__ double y[2 * kB], x[kB], res[kB], part[2 * kB];
     __shared__ int emax;
-    const int tid = threadIdx.x, i = tid & (kB - 1), h = tid >> 6, t = blockIdx.x;
+    const int tid = threadIdx.x, w = tid >> 5, t = blockIdx.x;
+    const int rt = w < 4 ? w : 7 - w;                                      // row tile; w and w + 4 share a scheduler
+    const int i = rt * 16 + (tid & 15), h = 2 * (w >> 2) + ((tid >> 4) & 1);  // row, column class (mod 4)
     const int64_t b = r0 / kB;
     const int f = upper ? kB : 0, s = kB - f;  // first and second half in the order of the substitution
     const int64_t bf = b + (upper ? 1 : 0), bs = b + (upper ? 0 : 1);
     const bool two = r0 + kB < N;  // the block has a second half
+    const bool first = !upper || two, second = two || upper;
+    const bool c1 = first && cond[2 * bf + upper] > kSolveCond, c2 = second && cond[2 * bs + upper] > kSolveCond;
     launch_dependents();
-    constexpr int kH = kB / 2;
-    double m1[kH], m2[kH], m3[kH];
-    auto load = [&](double(&m)[kH], bool on, const double *p) {
+    constexpr int kQ = kB / 4;  // columns of a thread
+    double v1[kQ], t1[kQ], o[kQ], v2[kQ], t2[kQ];
+    auto load = [&](double(&m)[kQ], bool on, const double *p) {
 #pragma unroll
-        for (int q = 0; q < kH; ++q) m[q] = on ? p[(h * kH + q) * kB + i] : 0.0;
+        for (int q = 0; q < kQ; ++q) m[q] = on ? p[(4 * q + h) * kB + i] : 0.0;
     };
-    load(m1, !upper || two, inv + (2 * bf + upper) * kB * kB);
-    load(m2, two, off + (2 * (b >> 1) + upper) * kB * kB);
-    load(m3, two || upper, inv + (2 * bs + upper) * kB * kB);
+    auto load_t = [&](double(&m)[kQ], bool on, int64_t rb) {  // the triangle at row rb
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) {
+            const int c = 4 * q + h;
+            const bool in = on && (upper ? c >= i : c < i) && rb + i < N && rb + c < N;
+            m[q] = in ? LU[(rb + i) * N + rb + c] : (!upper && c == i ? 1.0 : 0.0);
+        }
+    };
+    load(v1, first, inv + (2 * bf + upper) * kB * kB);
+    load_t(t1, c1, r0 + f);
+    load(o, two, off + (2 * (b >> 1) + upper) * kB * kB);
+    load(v2, second, inv + (2 * bs + upper) * kB * kB);
+    load_t(t2, c2, r0 + s);
     if (tid == 0) emax = 0;
     wait_dependencies();
-    y[tid] = t < T && r0 + tid < N ? Y[(r0 + tid) * T + t] : 0.0;
+    if (tid < 2 * kB) y[tid] = t < T && r0 + tid < N ? Y[(r0 + tid) * T + t] : 0.0;
     __syncthreads();
-    auto half_sum = [&](const double(&m)[kH], const double *v) {  // sum over this thread's half of the columns
-        double a[4] = {};
+    // row i of a product over the columns of the tiles [k0, k1); the two warps' parts are added up by the
+    // threads of h == 0
+    auto product = [&](const double(&m)[kQ], const double *v, int k0, int k1) {
+        double a0 = 0.0, a1 = 0.0;
 #pragma unroll
-        for (int q = 0; q < kH; q += 4)
+        for (int k = 0; k < 4; ++k) {
+            if (k < k0 || k >= k1) continue;  // warp-uniform
 #pragma unroll
-            for (int u = 0; u < 4; ++u) a[u] = fma(m[q + u], v[h * kH + q + u], a[u]);
-        part[tid] = (a[0] + a[1]) + (a[2] + a[3]);
+            for (int q = 4 * k; q < 4 * k + 4; q += 2) {
+                a0 = fma(m[q], v[4 * q + h], a0);
+                a1 = fma(m[q + 1], v[4 * q + 4 + h], a1);
+            }
+        }
+        double a = a0 + a1;
+        a += __shfl_xor_sync(0xffffffffu, a, 16);
+        if (!(h & 1)) part[(h >> 1) * kB + i] = a;
         __syncthreads();
     };
-    if (!upper || two) {
-        half_sum(m1, y + f);
-        if (h == 0) y[f + i] = part[i] + part[kB + i];
+    auto sum = [&] { return part[i] + part[kB + i]; };
+    const int k0 = upper ? rt : 0, k1 = upper ? 4 : rt + 1;  // a triangle's tiles
+    auto solve = [&](const double(&v)[kQ], const double(&m)[kQ], double *yh, bool correct) {
+        product(v, yh, k0, k1);
+        if (h == 0) (correct ? x : yh)[i] = sum();
         __syncthreads();
-    }
+        if (!correct) return;  // block-uniform
+        product(m, x, k0, k1);
+        if (h == 0) res[i] = yh[i] - sum();
+        __syncthreads();
+        product(v, res, k0, k1);
+        if (h == 0) yh[i] = x[i] + sum();
+        __syncthreads();
+    };
+    if (first) solve(v1, t1, y + f, c1);
     if (two) {
-        half_sum(m2, y + f);
-        if (h == 0) y[s + i] -= part[i] + part[kB + i];
+        product(o, y + f, 0, 4);
+        if (h == 0) y[s + i] -= sum();
         __syncthreads();
     }
-    if (two || upper) {
-        half_sum(m3, y + s);
-        if (h == 0) y[s + i] = part[i] + part[kB + i];
-        __syncthreads();
+    if (second) solve(v2, t2, y + s, c2);
+    if (tid < 2 * kB) {
+        const double v = r0 + tid < N ? y[tid] : 0.0;
+        if (t < T && r0 + tid < N) Y[(r0 + tid) * T + t] = v;
+        const int e = __reduce_max_sync(0xffffffffu, exp_field(v));
+        if ((tid & 31) == 0) atomicMax(&emax, e);
     }
-    const double v = r0 + tid < N ? y[tid] : 0.0;
-    if (t < T && r0 + tid < N) Y[(r0 + tid) * T + t] = v;
-    const int e = __reduce_max_sync(0xffffffffu, exp_field(v));
-    if ((tid & 31) == 0) atomicMax(&emax, e);
     __syncthreads();
     const int E = max(emax + 1, kEMin);
-    D[(int64_t)tid * Tp + t] = digits_of(v, E);
+    if (tid < 2 * kB) D[(int64_t)tid * Tp + t] = digits_of(r0 + tid < N ? y[tid] : 0.0, E);
     if (tid == 0) {
         Ex[t] = E;
         atomicMax(&Ex[Tp], E);
@@ -415,7 +477,8 @@ __global__ void __launch_bounds__(128) solve_diag(const double *__restrict__ inv
 // waiting for the one before: few rows a block, the factor's digits formed beside the kernel before, and,
 // where that leaves SMs idle, the inner dimension split over the warps (launch_update). N = 4,999, T = 9, a step (80 links, evaluation
 // 0.83 ms): 64-row blocks with a warp's whole inner dimension, each link after the one before 3.30 ms, now
-// 1.87; N = 10,242, T = 64 (160 links) 7.37 ms, with prologues beside the link before 6.89, now 4.20.
+// 1.89; N = 10,242, T = 64 (160 links) 7.37 ms, with prologues beside the link before 6.89, now 3.94 (4.20 before
+// solve_diag left out the triangles' empty tiles).
 constexpr int64_t kUpdateBlocks = 4 * 152;
 
 template <int KW>
@@ -627,7 +690,7 @@ int split_eval(const double *P, int64_t M, const double *X, int64_t K, int kind,
 
 size_t split_solve_factor_bytes(int64_t N) {
     const int64_t b = (N + kB - 1) / kB;
-    return (size_t)(2 * b + 2 * ((b + 1) / 2)) * kB * kB * sizeof(double);
+    return (size_t)(2 * b + 2 * ((b + 1) / 2)) * kB * kB * sizeof(double) + up256((size_t)2 * b * sizeof(double));
 }
 
 size_t split_solve_scratch_bytes(int64_t N, int T) {
@@ -637,17 +700,17 @@ size_t split_solve_scratch_bytes(int64_t N, int T) {
 
 int split_solve_prepare(const double *LU, int64_t N, void *factor, cudaStream_t s) {
     const int64_t b = (N + kB - 1) / kB;
-    double *inv = (double *)factor, *off = inv + 2 * b * kB * kB;
+    double *inv = (double *)factor, *off = inv + 2 * b * kB * kB, *cond = off + 2 * ((b + 1) / 2) * kB * kB;
     const int smem = 2 * kB * (kB + 1) * (int)sizeof(double);
     RBFSL_CUDA_TRY(cudaFuncSetAttribute(solve_prepare, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    solve_prepare<<<dim3((unsigned)b, 2), kB, smem, s>>>(LU, N, inv, off);
+    solve_prepare<<<dim3((unsigned)b, 2), kB, smem, s>>>(LU, N, inv, off, cond);
     return launch_status("global_solve prepare");
 }
 
 int split_solve(const double *LU, const int32_t *perm, int64_t N, const double *Q, int T, double *C, const void *factor,
                 void *scratch, cudaStream_t s) {
     const int64_t b64 = (N + kB - 1) / kB, b = (N + kChunk - 1) / kChunk;
-    const double *inv = (const double *)factor, *off = inv + 2 * b64 * kB * kB;
+    const double *inv = (const double *)factor, *off = inv + 2 * b64 * kB * kB, *cond = off + 2 * ((b64 + 1) / 2) * kB * kB;
     const int Tp = pad8(T);
     unsigned long long *D = (unsigned long long *)scratch;
     int *Ex = (int *)((char *)scratch + up256((size_t)kChunk * Tp * 8));  // one row per block step
@@ -657,7 +720,7 @@ int split_solve(const double *LU, const int32_t *perm, int64_t N, const double *
         const int upper = j >= b;
         const int64_t r0 = (upper ? 2 * b - 1 - j : j) * kChunk, nb = std::min<int64_t>(kChunk, N - r0);
         int *ex = Ex + j * (Tp + 1);
-        launch_after_prologue(solve_diag, dim3((unsigned)Tp), 128, 0, s, inv, off, N, r0, C, T, Tp, upper, D, ex);
+        launch_after_prologue(solve_diag, dim3((unsigned)Tp), 256, 0, s, LU, inv, off, cond, N, r0, C, T, Tp, upper, D, ex);
         const int64_t first = upper ? 0 : r0 + nb, rows = upper ? r0 : N - r0 - nb;
         if (rows <= 0) continue;
         const SrcF64 A{LU + first * N + r0, N};
