@@ -150,22 +150,33 @@ __device__ __forceinline__ double sqdist_rn(double ax, double ay, double az, dou
 // products of the high parts (FMA error term), the cross terms, and Knuth's two-sum into the
 // accumulator, so a step adds ~n 2^-48 relative rounding instead of the ~2^-24 of plain FP32.
 
-// v as a pair: hi = v to nearest (ties away from zero), lo = v - hi to nearest, by integer operations on
-// v's bits and one conversion of a 32-bit integer, because conversions between FP64 and FP32 run at the
-// FP64 rate. v = sign (1 + f) 2^e; 2^e is applied in two factors, which covers subnormal and zero results;
-// hi beyond FP32's range, infinite or NaN gives lo = NaN.
-__device__ __forceinline__ float2 pair_from(double v) {
+// v as a pair: hi = v to nearest, lo = v - hi to nearest, by integer operations on v's bits and one
+// conversion of a 32-bit integer, because conversions between FP64 and FP32 run at the FP64 rate.
+// v = sign (1 + f) 2^e; 2^e is applied in two factors, which covers subnormal and zero results (a lo below the
+// normal range is rounded twice). kStored, for values that are kept or returned: hi is what a conversion gives (ties to
+// even), NaN gives (NaN, NaN), an infinity (inf, NaN), a v that rounds beyond FP32's range (inf, -inf), with v's sign.
+// Without, for a factor on its way into a sum: ties go away from zero, and lo is NaN for all of these, hi an infinity
+// (the four operations less are 3% of the blend of partition-of-unity patches, 625 against 605 us a step at
+// N = 40,962, n = 84, T = 16).
+template <bool kStored>
+__device__ __forceinline__ float2 pair_split(double v) {
     const long long b = __double_as_longlong(v);
     const unsigned long long a = (unsigned long long)b & 0x7fffffffffffffffULL;
     const int field = (int)(a >> 52), e = min(max(field - 1023, -252), 128);
     const int f = (int)((a & 0xfffffffffffffULL) >> 28);          // the fraction's leading 24 bits
-    const int top = (f + 1) >> 1;                                 // 23 bits, rounded
-    const int rest = (int)(a & 0x1fffffffULL) - (f & 1 ? 1 << 29 : 0);  // the others, units of 2^(e - 52)
+    const int up = kStored ? f & ((f >> 1) | ((a & 0xfffffffULL) != 0)) & 1 : f & 1;
+    const int top = (f >> 1) + up;                                // 23 bits, rounded
+    const int rest = (int)(a & 0x1fffffffULL) - (up << 29);       // the others, units of 2^(e - 52)
     const int sign = (int)(b >> 32) & (int)0x80000000;
     const float s0 = __int_as_float(((e >> 1) + 127) << 23 | sign), s1 = __int_as_float((e - (e >> 1) + 127) << 23);
-    const float hi = __int_as_float(0x3f800000 + top) * s0 * s1;
-    return make_float2(hi, ((float)rest * 0x1p-52f) * s0 * s1 + (hi - hi));
+    float hi = __int_as_float(0x3f800000 + top) * s0 * s1, end = hi - hi;
+    if (kStored) {
+        if (a > 0x7ff0000000000000ULL) hi = end = __int_as_float(0x7fffffff);
+        else if (field < 0x7ff && fabsf(hi) == __int_as_float(0x7f800000)) end = -hi;
+    }
+    return make_float2(hi, ((float)rest * 0x1p-52f) * s0 * s1 + end);
 }
+__device__ __forceinline__ float2 pair_from(double v) { return pair_split<true>(v); }
 
 // (sh, sl) += w * q for pairs w and q; w.lo * q.lo (below 2^-48 |w q|) is dropped.
 __device__ __forceinline__ void pair_fma(float2 w, float2 q, float &sh, float &sl) {

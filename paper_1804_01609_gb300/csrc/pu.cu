@@ -594,9 +594,9 @@ template <>
 struct PuTerm<float2> {
     float h = 0.f, l = 0.f;
     static __device__ float2 factor(double dx, double dy, double dz, int half, double w) {
-        return pair_from(PuTerm<double>::factor(dx, dy, dz, half, w));
+        return pair_split<false>(PuTerm<double>::factor(dx, dy, dz, half, w));
     }
-    static __device__ float2 harmonic(double y, double w) { return pair_from(y * w); }
+    static __device__ float2 harmonic(double y, double w) { return pair_split<false>(y * w); }
     static __device__ float2 shfl(float2 v, int src) {
         return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
     }
