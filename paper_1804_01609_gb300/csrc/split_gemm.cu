@@ -27,16 +27,26 @@ namespace {
 
 constexpr int kChunk = kSplitChunk;
 constexpr int kLd = 136;  // shared row of a chunk's digits (16-byte loads of eight rows hit all banks)
-constexpr int kEMin = 64, kENan = 0x7ff;
+constexpr int kENan = 0x7ff;
 
-// ---- sources of A: raw 64-bit words, their exponent field, their digits, their value
+// The common exponent E of a row's or a column's chunk, |x| < 2^(E - 1023), from the largest key of its numbers (a
+// key grows with the magnitude): 2 for subnormal numbers, above kENan where one is not finite, in the middle of the
+// range for zeros, which are exact at any scale. A key of A's entries is their upper word alone (below 2^-1042 they
+// count as zeros), one operation for each.
+__device__ __forceinline__ int key_of(double x) {
+    return (__double2hiint(x) & 0x7fffffff) | (__double2loint(x) != 0);
+}
+__device__ __forceinline__ int chunk_exponent(int key) { return key == 0 ? 1024 : max(key >> 20, 1) + 1; }
+
+// ---- sources of A: raw 64-bit words, their keys, their digits, their value
 struct SrcF64 {
     const double *A;
     int64_t ld;
     __device__ __forceinline__ unsigned long long raw(int64_t r, int64_t k) const {
         return (unsigned long long)__double_as_longlong(A[r * ld + k]);
     }
-    __device__ __forceinline__ static int field(unsigned long long w) { return (int)(w >> 52) & 0x7ff; }
+    __device__ __forceinline__ static int key(unsigned long long w) { return (int)(w >> 32) & 0x7fffffff; }
+    __device__ __forceinline__ static int exponent(int key) { return chunk_exponent(key); }
     __device__ __forceinline__ static unsigned long long digits(unsigned long long w, int E) {
         return digits_of(__longlong_as_double((long long)w), E);
     }
@@ -60,9 +70,11 @@ struct SrcPair {
         const float2 v = A[r * ld + k];
         return (unsigned long long)__float_as_uint(v.x) | (unsigned long long)__float_as_uint(v.y) << 32;
     }
-    __device__ __forceinline__ static int field(unsigned long long w) {  // of the high part; not finite in either: kENan
-        const int e = (int)(w >> 23) & 0xff, f = (int)(w >> 55) & 0xff;
-        return e == 0xff || f == 0xff ? kENan : (e > f ? e : f) + 896;  // (a normalised pair has e >= f)
+    __device__ __forceinline__ static int key(unsigned long long w) {  // of the larger part
+        return max((int)w & 0x7fffffff, (int)(w >> 32) & 0x7fffffff);
+    }
+    __device__ __forceinline__ static int exponent(int key) {
+        return key == 0 ? 1024 : key >= 0x7f800000 ? kENan + 1 : (key >> 23) + 897;
     }
     __device__ __forceinline__ static unsigned long long digits(unsigned long long w, int E) {
         return (unsigned long long)(fixed_of((uint32_t)w, E) + fixed_of((uint32_t)(w >> 32), E)) + 0x8080808080808080ULL;
@@ -86,9 +98,15 @@ struct SrcPhi : SrcF64 {
 __device__ __forceinline__ double x_value(const double *x) { return *x; }
 __device__ __forceinline__ double x_value(const float2 *x) { return (double)x->x + (double)x->y; }
 
+constexpr int kExtra = 2, kExTop = 4096;  // entries behind a chunk's exponents
+__device__ __forceinline__ void column_extremes(int *e, int E) {
+    atomicMax(e, E);
+    atomicMax(e + 1, kExTop - E);
+}
+
 // Digits of x (K x T, row-major), chunk blockIdx.x, columns blockIdx.y * 32 .. + 32: D[chunk][k][t]
-// (row length Tp), the columns' exponents Ex[chunk][t] (largest field + 1, at least kEMin; not finite:
-// above kENan) and their largest, Ex[chunk][Tp] (zeroed by the caller).
+// (row length Tp), the columns' exponents Ex[chunk][t] (chunk_exponent), their largest, Ex[chunk][Tp], and
+// kExTop less their smallest, Ex[chunk][Tp + 1] (zeroed by the caller).
 template <typename V>
 __global__ void __launch_bounds__(256) x_digits(const V *__restrict__ x, int64_t K, int T, int Tp,
                                                 unsigned long long *__restrict__ D, int *__restrict__ Ex) {
@@ -103,28 +121,35 @@ __global__ void __launch_bounds__(256) x_digits(const V *__restrict__ x, int64_t
     for (int u = 0; u < kChunk / 8; ++u) {
         const int64_t k = k0 + w + 8 * u;
         v[u] = k < K && t < T ? x_value(x + k * T + t) : 0.0;
-        e = max(e, exp_field(v[u]));
+        e = max(e, key_of(v[u]));
     }
     atomicMax(&emax[c], e);
     __syncthreads();
-    const int E = max(emax[c] + 1, kEMin);
+    const int E = chunk_exponent(emax[c]);
     if (t < Tp) {
 #pragma unroll
         for (int u = 0; u < kChunk / 8; ++u) D[(k0 + w + 8 * u) * Tp + t] = digits_of(v[u], E);
         if (w == 0) {
-            Ex[ch * (Tp + 1) + t] = E;
-            atomicMax(&Ex[ch * (Tp + 1) + Tp], E);
+            int *ex = Ex + ch * (Tp + kExtra);
+            ex[t] = E;
+            column_extremes(ex + Tp, E);
         }
     }
 }
 
-// Scale of a chunk's sums: 2^(EA + EX - 2 * 1023 - 34), 0 where it is below the normal doubles.
+// Scale of a chunk's sums, 2^(EA + EX - 2 * 1023 - 34), and whether it is a normal double.
+__device__ __forceinline__ bool chunk_tiny(int EA, int EX) { return EA + EX <= 1023 + 34; }
 __device__ __forceinline__ double chunk_scale(int EA, int EX) {
-    const int e = EA + EX - 1023 - 34;
-    return __longlong_as_double((long long)(e > 0 ? e : 0) << 52);
+    return __longlong_as_double((long long)(EA + EX - 1023 - 34) << 52);
+}
+// v times that scale for any EA and EX, in two factors (0 for one below the normal doubles: v < 2^62). The
+// second of two paths: a warp takes it where one of its scales may not be a normal double.
+__device__ __forceinline__ double chunk_scaled(double v, int EA, int EX) {
+    const int X = EA + EX - 2 * 1023 - 34, a = X >> 1, b = X - a;
+    return v * __longlong_as_double((long long)max(a + 1023, 0) << 52) * __longlong_as_double((long long)max(b + 1023, 0) << 52);
 }
 
-// Whether a chunk's sums need plain FP64: rows (2 kENan) or columns that are not finite, or results beyond
+// Whether a chunk's sums need plain FP64: rows or columns that are not finite, or results beyond
 // the doubles' range.
 __device__ __forceinline__ bool chunk_bad(int ea_max, int ex_max) {
     return ea_max > kENan || ex_max > kENan || ea_max + ex_max >= 2047 + 1023 + 34;
@@ -149,7 +174,8 @@ __global__ void __launch_bounds__(128, 3) split_gemm_kernel(Src A, int64_t M, in
         const int kc = (int)min((int64_t)kChunk, K - k0);
         // ---- digits of the block's rows, four rows of a warp at a time
         bool bad = false;
-        const int exm = Ex[(int64_t)ch * (Tp + 1) + Tp];
+        const int *ex = Ex + (int64_t)ch * (Tp + kExtra);
+        const int exm = ex[Tp], exs = kExTop - ex[Tp + 1];
         for (int q = 0; q < kRows / 4; q += 4) {
             unsigned long long w[4][4];
 #pragma unroll
@@ -166,11 +192,10 @@ __global__ void __launch_bounds__(128, 3) split_gemm_kernel(Src A, int64_t M, in
                 const int row = warp * (kRows / 4) + q + v;
                 int e = 0;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) e = max(e, Src::field(w[v][u]));
-                e = __reduce_max_sync(0xffffffffu, e);
-                const int E = max(e + 1, kEMin);
+                for (int u = 0; u < 4; ++u) e = max(e, Src::key(w[v][u]));
+                const int E = Src::exponent(__reduce_max_sync(0xffffffffu, e));
                 if (lane == 0) Er[row] = E;
-                bad |= chunk_bad(e >= kENan ? 2 * kENan : E, exm);
+                bad |= chunk_bad(E, exm);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) As[row * kLd + lane + 32 * u] = Src::digits(w[v][u], E);
             }
@@ -189,6 +214,8 @@ __global__ void __launch_bounds__(128, 3) split_gemm_kernel(Src A, int64_t M, in
                             sum[nt][u] = fma(Src::value(A.raw(r, k0 + k)), x_value(x + (k0 + k) * T + t), sum[nt][u]);
                 }
         } else {
+            const int ea[2] = {Er[wr + g], Er[wr + g + 8]};
+            const bool tiny = __any_sync(0xffffffffu, chunk_tiny(min(ea[0], ea[1]), exs));
 #pragma unroll
             for (int np = 0; np < 2; ++np) {  // two 8-column tiles at a time
                 const int cb = col0 + 16 * np;
@@ -229,11 +256,17 @@ __global__ void __launch_bounds__(128, 3) split_gemm_kernel(Src A, int64_t M, in
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     if (h == 1 && !two) break;
+                    const int et[2] = {ex[cb + 8 * h + t2], ex[cb + 8 * h + t2 + 1]};
+                    if (!tiny) {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int ea = Er[wr + g + 8 * (u >> 1)],
-                                  ex = Ex[(int64_t)ch * (Tp + 1) + cb + 8 * h + t2 + (u & 1)];
-                        sum[2 * np + h][u] = fma(split_value(acc[h], u), chunk_scale(ea, ex), sum[2 * np + h][u]);
+                        for (int u = 0; u < 4; ++u)
+                            sum[2 * np + h][u] = fma(split_value(acc[h], u), chunk_scale(ea[u >> 1], et[u & 1]),
+                                                     sum[2 * np + h][u]);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            sum[2 * np + h][u] += chunk_scaled(split_value(acc[h], u), ea[u >> 1], et[u & 1]);
+                        __syncwarp();
                     }
                 }
             }
@@ -460,15 +493,15 @@ __global__ void __launch_bounds__(256, 1) solve_diag(const double *__restrict__ 
     if (tid < 2 * kB) {
         const double v = r0 + tid < N ? y[tid] : 0.0;
         if (t < T && r0 + tid < N) Y[(r0 + tid) * T + t] = v;
-        const int e = __reduce_max_sync(0xffffffffu, exp_field(v));
+        const int e = __reduce_max_sync(0xffffffffu, key_of(v));
         if ((tid & 31) == 0) atomicMax(&emax, e);
     }
     __syncthreads();
-    const int E = max(emax + 1, kEMin);
+    const int E = chunk_exponent(emax);
     if (tid < 2 * kB) D[(int64_t)tid * Tp + t] = digits_of(r0 + tid < N ? y[tid] : 0.0, E);
     if (tid == 0) {
         Ex[t] = E;
-        atomicMax(&Ex[Tp], E);
+        column_extremes(Ex + Tp, E);
     }
 }
 
@@ -477,7 +510,7 @@ __global__ void __launch_bounds__(256, 1) solve_diag(const double *__restrict__ 
 // waiting for the one before: few rows a block, the factor's digits formed beside the kernel before, and,
 // where that leaves SMs idle, the inner dimension split over the warps (launch_update). N = 4,999, T = 9, a step (80 links, evaluation
 // 0.83 ms): 64-row blocks with a warp's whole inner dimension, each link after the one before 3.30 ms, now
-// 1.89; N = 10,242, T = 64 (160 links) 7.37 ms, with prologues beside the link before 6.89, now 3.94 (4.20 before
+// 1.88; N = 10,242, T = 64 (160 links) 7.37 ms, with prologues beside the link before 6.89, now 4.02 (4.20 before
 // solve_diag left out the triangles' empty tiles).
 constexpr int64_t kUpdateBlocks = 4 * 152;
 
@@ -507,11 +540,10 @@ __global__ void __launch_bounds__(128, 3) solve_update(SrcF64 A, int64_t M, int 
         for (int v = 0; v < 4; ++v) {
             int e = 0;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) e = max(e, SrcF64::field(w[v][u]));
-            e = __reduce_max_sync(0xffffffffu, e);
-            const int E = max(e + 1, kEMin);
+            for (int u = 0; u < 4; ++u) e = max(e, SrcF64::key(w[v][u]));
+            const int E = SrcF64::exponent(__reduce_max_sync(0xffffffffu, e));
             if (lane == 0) Er[4 * warp + v] = E;
-            ea_max = max(ea_max, e >= kENan ? 2 * kENan : E);
+            ea_max = max(ea_max, E);
 #pragma unroll
             for (int u = 0; u < 4; ++u) As[(4 * warp + v) * kLd + lane + 32 * u] = SrcF64::digits(w[v][u], E);
         }
@@ -557,13 +589,24 @@ __global__ void __launch_bounds__(128, 3) solve_update(SrcF64 A, int64_t M, int 
                 split_products(acc[1], av, b);
             }
         }
+        const int ea[2] = {Er[g], Er[g + 8]};
+        const bool tiny = __any_sync(0xffffffffu, chunk_tiny(min(ea[0], ea[1]), kExTop - Ex[Tp + 1]));
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1 && !two) break;
+            const int t = cb + 8 * h + t2, et[2] = {Ex[t], Ex[t + 1]};
+            double *o = &part[kw][g * kCols + t - col0];
+            if (!tiny) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int r = g + 8 * (u >> 1), t = cb + 8 * h + t2 + (u & 1);
-                if (h == 0 || two) part[kw][r * kCols + t - col0] = split_value(acc[h], u) * chunk_scale(Er[r], Ex[t]);
+                for (int u = 0; u < 4; ++u)
+                    o[8 * kCols * (u >> 1) + (u & 1)] = split_value(acc[h], u) * chunk_scale(ea[u >> 1], et[u & 1]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    o[8 * kCols * (u >> 1) + (u & 1)] = chunk_scaled(split_value(acc[h], u), ea[u >> 1], et[u & 1]);
+                __syncwarp();
             }
+        }
     }
     __syncthreads();
 #pragma unroll
@@ -643,7 +686,7 @@ Plan plan(int64_t M, int64_t K, int T, bool direct) {
         }
     }
     p.digits = up256((size_t)nchunk * kChunk * pad8(T) * 8);
-    p.exps = up256((size_t)nchunk * (pad8(T) + 1) * sizeof(int));
+    p.exps = up256((size_t)nchunk * (pad8(T) + kExtra) * sizeof(int));
     p.part = p.splits > 1 || !direct ? (size_t)p.splits * M * T * sizeof(double) : 0;
     return p;
 }
@@ -695,7 +738,7 @@ size_t split_solve_factor_bytes(int64_t N) {
 
 size_t split_solve_scratch_bytes(int64_t N, int T) {
     const int64_t b = (N + kChunk - 1) / kChunk;
-    return up256((size_t)kChunk * pad8(T) * 8) + (size_t)2 * b * (pad8(T) + 1) * sizeof(int);
+    return up256((size_t)kChunk * pad8(T) * 8) + (size_t)2 * b * (pad8(T) + kExtra) * sizeof(int);
 }
 
 int split_solve_prepare(const double *LU, int64_t N, void *factor, cudaStream_t s) {
@@ -714,12 +757,12 @@ int split_solve(const double *LU, const int32_t *perm, int64_t N, const double *
     const int Tp = pad8(T);
     unsigned long long *D = (unsigned long long *)scratch;
     int *Ex = (int *)((char *)scratch + up256((size_t)kChunk * Tp * 8));  // one row per block step
-    RBFSL_CUDA_TRY(cudaMemsetAsync(Ex, 0, (size_t)2 * b * (Tp + 1) * sizeof(int), s));
+    RBFSL_CUDA_TRY(cudaMemsetAsync(Ex, 0, (size_t)2 * b * (Tp + kExtra) * sizeof(int), s));
     solve_gather<<<(unsigned)((N * T + 255) / 256), 256, 0, s>>>(Q, perm, N, T, C);
     for (int64_t j = 0; j < 2 * b; ++j) {
         const int upper = j >= b;
         const int64_t r0 = (upper ? 2 * b - 1 - j : j) * kChunk, nb = std::min<int64_t>(kChunk, N - r0);
-        int *ex = Ex + j * (Tp + 1);
+        int *ex = Ex + j * (Tp + kExtra);
         launch_after_prologue(solve_diag, dim3((unsigned)Tp), 256, 0, s, LU, inv, off, cond, N, r0, C, T, Tp, upper, D, ex);
         const int64_t first = upper ? 0 : r0 + nb, rows = upper ? r0 : N - r0 - nb;
         if (rows <= 0) continue;
