@@ -210,15 +210,24 @@ int rbfsl_global_factor_chol(const double *x, int64_t N, int kernel, double eps,
                              int32_t *perm, void *stream);
 
 /* Coefficients of the global interpolant for T fields: solve A_X c = q with the factor of
- * rbfsl_global_factor or rbfsl_global_factor_chol (forward and backward substitution, FP64).
+ * rbfsl_global_factor or rbfsl_global_factor_chol by forward and backward substitution in blocks,
+ * to FP64 accuracy. Two forms: FP64 throughout, in 64-row blocks; or, for N >= 384 or N T >= 98,304 (N > 64), 128-row
+ * blocks with the inverses of their 64-row halves (each product corrected once where the block's condition
+ * asks for it) and the updates as digit products on the tensor cores. The second takes stream-ordered scratch
+ * for the call (cudaMallocAsync on `stream`, freed on it; 1.5 kB a row, 1 kB + N / 16 bytes a tracer);
+ * under stream capture, or where there is no memory for it, the first runs for any size and the
+ * result differs by rounding.
  * q, c: device N x T, may not alias. Errors: EINVAL, ECUDA. */
 int rbfsl_global_solve(const double *LU, const int32_t *perm, int64_t N, const double *q, int T,
                        double *c, void *stream);
 
 /* Evaluate the global interpolant (Eq. srbfinterp) at Nq points for T fields:
  *   out[i][t] = sum_j phi(|p_i - x_j|) c[j][t].
- * dtype RBFSL_F64: c and out FP64, FP64 arithmetic. RBFSL_F32: c and out FP32, FP32 kernel
- * values and FP32 accumulation (the mixed-precision evaluation).
+ * dtype RBFSL_F64: c and out FP64; kernel values in FP64, the products in FP64 or, for N >= 384 or
+ * Nq N ceil(T / 64) >= 1,500,000, to FP64 accuracy as digit products on the tensor cores, with
+ * stream-ordered scratch for the call as in rbfsl_global_solve (the digits of c, 8 bytes a value, and partial
+ * sums of up to 32 times the result); without it (capture, no memory) FP64 products. RBFSL_F32: c and out FP32,
+ * FP32 kernel values and FP32 accumulation (the mixed-precision evaluation).
  * p: device Nq x 3, x: device N x 3. Errors: EINVAL, ECUDA. */
 int rbfsl_global_eval(const double *p, int64_t Nq, const double *x, int64_t N, int kernel,
                       double eps, const void *c, int T, int dtype, void *out, void *stream);

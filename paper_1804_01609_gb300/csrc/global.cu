@@ -473,10 +473,16 @@ struct Scratch {
 
 }  // namespace
 
-// C = A_X^-1 Q, the solve's blocks inverted and its scratch taken for this call; systems of one
-// 64-row block have no trailing update to gain from.
+// Where a call's scratch costs more than the digit products save. A call whose stream is waited for after
+// each pays ~130 us for its allocation (the pool gives its memory back) and ~60 more for inverting a solve's blocks. Solve, microseconds
+// without and with scratch: N = 128 115 / 261, 257 274 / 358, 320 317 / 334, 384 384 / 352, 642 672 / 380
+// (T = 1; the same up to 64 tracers); T = 512: N = 192 550 / 454, 257 883 / 566. Evaluation, T = 4, N = Nq = 128 73 / 167, 257 nodes
+// and 1,000 points 148 / 169, 384 nodes 193 / 170; 128 nodes and 5,000 points 121 / 163, 10,000 214 / 193.
+constexpr int64_t kScratchNodes = 384, kScratchSolve = 96 * 1024, kScratchEval = 1500000;
+
+// C = A_X^-1 Q, the solve's blocks inverted and its scratch taken for this call.
 int global_solve(const double *LU, const int32_t *perm, int64_t N, const double *Q, int T, double *C, cudaStream_t s) {
-    if (N > kNb) {
+    if (N >= kScratchNodes || (N > kNb && N * T >= kScratchSolve)) {
         const size_t fb = split_solve_factor_bytes(N);
         Scratch ws(fb + split_solve_scratch_bytes(N, T), s);
         if (ws.p) {
@@ -563,8 +569,10 @@ int launch_global_eval(const double *P, int64_t Nq, const double *X, int64_t N, 
     dim3 grid((unsigned)((Nq + 31) / 32), (unsigned)((T + 63) / 64));
     const double e2 = eps * eps;
     if (dtype == RBFSL_F64) {
-        Scratch ws(split_product_bytes(Nq, N, T, RBFSL_F64), s);
-        if (ws.p) return split_eval(P, Nq, X, N, kind, eps, (const double *)C, T, RBFSL_F64, out, ws.p, s);
+        if (N >= kScratchNodes || Nq * N * grid.y >= kScratchEval) {
+            Scratch ws(split_product_bytes(Nq, N, T, RBFSL_F64), s);
+            if (ws.p) return split_eval(P, Nq, X, N, kind, eps, (const double *)C, T, RBFSL_F64, out, ws.p, s);
+        }
         // without scratch, FP64 products: 8 points per block (64 threads): four times the blocks of 32, so that the FP64-bound
         // grid spreads evenly over the SMs (N = 10,242: 1,281 blocks instead of 321; 22.4 ->
         // 18.0 ms at T = 64)
