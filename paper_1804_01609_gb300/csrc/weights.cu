@@ -69,8 +69,9 @@ struct WeightsArgs {
 // the group barrier is __syncwarp; with NW > 1 a block is one point and uses __syncthreads. kBlocks:
 // the blocks per SM that the registers are bounded for: seven for one warp per point (72 registers);
 // with two and four warps, whose digit products want 117 to 128, what shared memory allows (eight points of
-// two warps, five or four of four).
-template <int NW, int kBlocks, typename WT>
+// two warps, five or four of four). kReduced: whether the kernel serves the reduced form; without, the
+// indefinite factorisation alone, in 72 registers.
+template <int NW, int kBlocks, bool kReduced, typename WT>
 __global__ void __launch_bounds__(NW == 2 ? 64 : 128, kBlocks) weights_kernel(WeightsArgs a, WT *__restrict__ W) {
     extern __shared__ double smem[];
     constexpr int GT = NW * kWarp;
@@ -80,18 +81,23 @@ __global__ void __launch_bounds__(NW == 2 ? 64 : 128, kBlocks) weights_kernel(We
     if (i >= a.Nq) return;  // NW == 1 only (with NW > 1 the grid has exactly Nq blocks)
     double *R = smem + (size_t)g * a.region_doubles;
     double *w = nullptr;
-    const int rc = weights_point<NW, NW != 1>(R, a.X, a.idx + i * a.n, a.n, a.m, a.ell, a.half,
-                                         a.P[3 * i], a.P[3 * i + 1], a.P[3 * i + 2], t, w);
+    int rc;
+    if constexpr (kReduced)
+        rc = weights_point<NW, NW != 1>(R, a.X, a.idx + i * a.n, a.n, a.m, a.ell, a.half, a.P[3 * i], a.P[3 * i + 1],
+                                        a.P[3 * i + 2], t, w);
+    else
+        rc = weights_point_ldl<NW>(R, a.X, a.idx + i * a.n, a.n, a.m, a.ell, a.half, a.P[3 * i], a.P[3 * i + 1],
+                                   a.P[3 * i + 2], t, w);
     if (t >= kWarp) return;
     const int n = a.n, lane = t;
     for (int j = lane; j < n; j += kWarp) W[i * n + j] = wcast<WT>(rc == RBFSL_OK ? w[j] : (double)NAN);
     if (a.status && lane == 0) a.status[i] = rc;
 }
 
-template <int NW, int kBlocks, typename WT>
+template <int NW, int kBlocks, bool kReduced, typename WT>
 int launch_weights_nw(const WeightsArgs &a, int spb, void *w, cudaStream_t s) {
     const int smem = spb * a.region_doubles * 8;
-    auto *kernel = weights_kernel<NW, kBlocks, WT>;
+    auto *kernel = weights_kernel<NW, kBlocks, kReduced, WT>;
     RBFSL_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     // all of the unified L1 / shared storage as shared memory: as many points per SM as fit
     RBFSL_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
@@ -100,11 +106,11 @@ int launch_weights_nw(const WeightsArgs &a, int spb, void *w, cudaStream_t s) {
     return launch_status("stencil_weights");
 }
 
-template <int NW, int kBlocks>
+template <int NW, int kBlocks, bool kReduced = true>
 int launch_weights_typed(const WeightsArgs &a, int spb, void *w, int w_dtype, cudaStream_t s) {
-    if (w_dtype == RBFSL_F64) return launch_weights_nw<NW, kBlocks, double>(a, spb, w, s);
-    if (w_dtype == RBFSL_F32X2) return launch_weights_nw<NW, kBlocks, float2>(a, spb, w, s);
-    return launch_weights_nw<NW, kBlocks, float>(a, spb, w, s);
+    if (w_dtype == RBFSL_F64) return launch_weights_nw<NW, kBlocks, kReduced, double>(a, spb, w, s);
+    if (w_dtype == RBFSL_F32X2) return launch_weights_nw<NW, kBlocks, kReduced, float2>(a, spb, w, s);
+    return launch_weights_nw<NW, kBlocks, kReduced, float>(a, spb, w, s);
 }
 
 int launch_weights(const double *x, const int32_t *idx, int64_t Nq, int n, int ell, int power,
@@ -118,7 +124,13 @@ int launch_weights(const double *x, const int32_t *idx, int64_t Nq, int n, int e
     a.m = n + (ell + 1) * (ell + 1);
     a.region_doubles = weights_doubles(n, a.m, ell, a.half);
     const int bytes = a.region_doubles * 8;
-    if (bytes > kWeightsSmallBytes || (reduced_form(n, ell, a.half) && reduced_on_tensor(a.m - n))) {
+    const bool reduced = reduced_form(n, ell, a.half);
+    // the indefinite factorisation's steps are all block-wide: four warps per point, and registers for the six or
+    // seven points that an SM holds up to 37 KB a point (m = 54 at N = 2,562 488 us, two warps 536; m = 81 at N =
+    // 12,347 4.26 ms, bounded for five points 4.72)
+    if (!reduced && bytes > kWeightsSmallBytes && bytes <= 37 * 1024)
+        return launch_weights_typed<4, 7, false>(a, 1, w, w_dtype, s);
+    if (bytes > kWeightsSmallBytes || (reduced && reduced_on_tensor(a.m - n))) {
         // larger systems (m >~ 45, or with the products on the tensor cores), one point per block: two warps
         // per point while eight points fit an SM's 227 KB (more points overlap each other's serial steps:
         // m = 71 at N = 12,347 1.73 ms, four warps and five points 1.90), else four warps; five blocks need
