@@ -490,7 +490,7 @@ typedef struct rbfsl_server_info_t {
     double now_s;
 } rbfsl_server_info_t;
 /* budget: device bytes the running requests may hold together (admission estimate per request:
- * nodes, departure points, fields, index, stencil or patch factors). max_slots: concurrent
+ * nodes, departure points, fields, index, stencil or patch factors and their set-up). max_slots: concurrent
  * requests. Starts the scheduler thread. Errors: EINVAL, ECUDA, ENOMEM. */
 int rbfsl_server_create(rbfsl_server **out, int device, size_t hbm_budget_bytes, int max_slots);
 /* Stop the scheduler and free everything (running requests are dropped). */

@@ -187,6 +187,8 @@ int pu_apply_begin(rbfsl_pu *u, const void *q, int q_dtype, int T, int dtype, cu
 int pu_apply_end(rbfsl_pu *u, int T, const double *p, int64_t Nq, int wkind, int dtype, void *out, int32_t *status,
                  cudaStream_t s);
 
+size_t pu_estimate_bytes(int64_t N, int64_t Mp, int members, int ell, int power, int T);
+
 int launch_stencil_factor(const double *X, const int64_t *mstart, const int32_t *members,
                           const int64_t *lu_off, int64_t count, int max_n, int M, int ell,
                           int power, double *LU, int32_t *perm, int32_t *status, cudaStream_t s,

@@ -813,13 +813,28 @@ void pu_free(rbfsl_pu *u) {
     cudaFree(u->pt_cnt); cudaFree(u->pt_id); cudaFree(u->pt_w); cudaFree(u->pt_Y);
 }
 
-// Reduced factors of every patch, packed from a scratch buffer of at most ~256 MB at a time. Returns 1
+constexpr int64_t kPuPackBytes = (int64_t)64 << 20;  // of unpacked factors at a time
+
+// Device bytes of a handle and its set-up for Mp patches of at most `members` nodes each, T tracers.
+size_t pu_estimate_bytes(int64_t N, int64_t Mp, int members, int ell, int power, int T) {
+    const int M = (ell + 1) * (ell + 1), m = members + M;
+    double factor = 8.0 * m * m, scratch = 0.0;  // LU, where a patch has no reduced form
+    if (reduced_form(members, ell, (power - 1) / 2)) {
+        factor = std::max(factor, 8.0 * PatchLayout(members, M).total);
+        scratch = std::min((double)kPuPackBytes, 8.0 * Mp * CenterLayout(members, M).total);
+    }
+    const double points = (double)std::min(std::max(N, kPuMinChunk), kPuMaxChunk);
+    return (size_t)(N * (3 * 8.0 + 28.0) + Mp * (factor + m * (36.0 + 8.0 * T) + 24 + 28 + 24) + scratch +
+                    points * (4 + kPuMaxPatches * 12 + M * 8));
+}
+
+// Reduced factors of every patch, packed from a scratch buffer of at most kPuPackBytes at a time. Returns 1
 // (with nothing kept) where a patch has none: its reduced matrix breaks down or its nodes coincide.
 int pu_build_reduced(rbfsl_pu *u, const std::vector<int64_t> &ms, const std::vector<int32_t> &hc, int half,
                      cudaStream_t s) {
     const int M = u->M;
     const int64_t Mp = u->Mp, stride = CenterLayout(u->max_members, M).total;
-    const int64_t chunk = std::min<int64_t>(Mp, std::max<int64_t>(1, ((int64_t)256 << 20) / (stride * 8)));
+    const int64_t chunk = std::min<int64_t>(Mp, std::max<int64_t>(1, kPuPackBytes / (stride * 8)));
     std::vector<int64_t> off(Mp);
     int64_t total = 0;
     for (int64_t l = 0; l < Mp; ++l) {

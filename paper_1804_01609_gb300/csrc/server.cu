@@ -8,6 +8,7 @@
 //   3. retire requests that reached their step count (copy the field out, free the memory,
 //      record the latency).
 // Node sets, stencil state and fields stay on the device between steps.
+#include <algorithm>
 #include <chrono>
 #include <cstdio>
 #include <string>
@@ -51,8 +52,9 @@ struct Req {
     std::string err;
 };
 
-// Device bytes a request holds while it runs (nodes, departure points, status, two fields,
-// grid index, stencil factors or patch factors).
+// Device bytes a request holds while it runs or is set up (nodes, departure points, status, two fields,
+// grid index, stencil factors or patch factors). Centre stencils: LU factors, which are kept where a stencil has no
+// reduced form and are the larger of the two.
 size_t estimate_bytes(const rbfsl_request &r) {
     const double N = (double)r.problem.N, T = r.problem.T;
     const double es = 8.0;  // FP64 or FP32-pair weights
@@ -65,8 +67,9 @@ size_t estimate_bytes(const rbfsl_request &r) {
     } else {
         const double R = r.pu_radius > 0 ? r.pu_radius : 2.0 * std::sqrt(r.problem.n / N);
         const double per = N * R * R / 4.0 * 1.3;  // nodes per patch, with margin
-        const double m = per + M;
-        b += (double)r.pu_Mp * (m * m * 8.0 + m * 4.0 + m * T * 12.0) + N * T * 8.0;
+        const int members = per > 0.0 ? (int)std::ceil(std::min(per, (double)RBFSL_MAX_SYSTEM)) : 1;
+        b += (double)pu_estimate_bytes(r.problem.N, r.pu_Mp, members, r.problem.ell, (int)r.problem.phs_power,
+                                       r.problem.T);
     }
     return (size_t)b;
 }
