@@ -289,7 +289,7 @@ __device__ __forceinline__ bool key_less(long long da, int ia, long long db, int
 // k nearest nodes of (qx, qy, qz) by one warp. bd/bi: the warp's candidate buffers (cap
 // entries, cap a power of two >= k). On success bi[0..k) holds the node indices ascending by
 // (d2, index) and the function returns true; false if no radius in 40 rescalings brackets between
-// k and cap candidates. A single neighbour is kept in registers instead of a sorted list. The radius of
+// k and cap candidates (more than cap - k nodes at one distance). A single neighbour is kept in registers instead of a sorted list. The radius of
 // the cells' tests in FP32 (the FP64 root and its conversions were a third of the FP64 instructions of a
 // k = 1 query): 249 -> 143 us at N = 163,842, k = 1; 218 -> 204 us at N = 40,962, k = 84.
 __device__ __forceinline__ bool knn_warp(const KnnGrid &g, double qx, double qy, double qz, int k,
@@ -297,6 +297,7 @@ __device__ __forceinline__ bool knn_warp(const KnnGrid &g, double qx, double qy,
     // a ball that holds 1.3 k nodes on average; few neighbours take three more, so that the first
     // ball is seldom empty
     double r2 = g.r2_per_k * (k < 16 ? k + 3 : k);
+    double lo = 0.0, hi = INFINITY;  // the largest radius (squared) with too few, the smallest with too many
     const double target = 1.3 * k;
     const unsigned below = (1u << lane) - 1u;
     int total = 0;
@@ -333,12 +334,16 @@ __device__ __forceinline__ bool knn_warp(const KnnGrid &g, double qx, double qy,
             ok = true;
             break;
         }
-        // Rescale the radius towards ~1.3 k candidates (count grows like r^2).
+        // Rescale the radius towards ~1.3 k candidates (count grows like r^2), by halves once that leaves the
+        // bracket: where the density varies, rescaling alone can go back and forth over it.
+        if (total < k) lo = r2;
+        else hi = r2;
         double f = total > 0 ? target / (double)total : 4.0;
         f = f < 0.25 ? 0.25 : (f > 4.0 ? 4.0 : f);
         if (total < k && f < 1.05) f = 1.05;
         if (total > cap && f > 0.95) f = 0.95;
         r2 *= f;
+        if (r2 <= lo || r2 >= hi) r2 = 0.5 * (lo + hi);
     }
     if (!ok) return false;
     if (k == 1) {
