@@ -31,7 +31,7 @@ namespace rbfsl {
 
 struct BatchDesc {
     int64_t N;
-    int n, ell, half, m, ld, T;
+    int n, ell, half, m, T;
     int mode, mixed, ppt, active;
     int vel_kind;
     double vel[4];   // as given (kernel-ready forms are built on the device)
@@ -548,7 +548,7 @@ int rbfsl_batch_add(rbfsl_batch *b, const rbfsl_problem *pr, int *id_out) {
     }
     RBFSL_CUDA_TRY(cudaStreamSynchronize(s));
     BatchDesc &d = h.d;
-    d.N = N; d.n = (int)n; d.ell = pr->ell; d.half = (pw - 1) / 2; d.m = m; d.ld = (m + 1) | 1; d.T = pr->T;
+    d.N = N; d.n = (int)n; d.ell = pr->ell; d.half = (pw - 1) / 2; d.m = m; d.T = pr->T;
     d.mode = pr->mode; d.mixed = pr->precision == RBFSL_MIXED; d.active = 1;
     d.vel_kind = pr->vel_kind;
     for (int i = 0; i < 4; ++i) d.vel[i] = pr->vel_params[i];

@@ -83,10 +83,6 @@ struct CenterLayout {
     }
     __host__ __device__ int fold(int i, int j) const { return i < H ? j * H + i : (j + K - i) * H + K - 1 - i; }
 };
-__host__ __device__ inline int center_factor_doubles(int n, int ell, int half) {
-    const int M = (ell + 1) * (ell + 1);
-    return reduced_form(n, ell, half) ? CenterLayout(n, M).total : (n + M) * (n + M);
-}
 
 // Shared doubles of one point: the reduced form's region or the indefinite factorisation's (the
 // path of systems without the reduced form, and of a point whose reduced matrix breaks down),
