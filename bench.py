@@ -10,7 +10,8 @@ precision = FP64 solves, FP32 stage increments in the tracer, weights and fields
 with the W.q sum in pair arithmetic.
 
 The L2 cache (129 MB) is flushed between timed steps by writing a 256 MB buffer, so every
-step starts cold. Prints one JSON line (rank 0).
+step starts cold. Prints one JSON line (rank 0); the full record of every leg goes to stderr, or to
+the file given by --record.
 """
 from __future__ import annotations
 
@@ -51,6 +52,7 @@ def parse():
                     help="run one kernel of the workload on --nq points (for profilers); no JSON")
     ap.add_argument("--nq", type=int, default=3040)
     ap.add_argument("--repeat", type=int, default=3)
+    ap.add_argument("--record", default=None, metavar="FILE", help="write the full record here instead of to stderr")
     return ap.parse_args()
 
 
@@ -156,6 +158,10 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # capture (dram__bytes_read.sum + dram__bytes_write.sum) of the kernel version this file ships
 # with; None when no capture of that version exists.
 WEIGHTS_DRAM_BYTES = 16.4e6
+# FP64 warp instructions per point of that kernel at m = 109, from the same capture
+# (sm__inst_executed_pipe_fp64.sum = 2.18e8 for 40,962 points): the FP64 pipe's work, whatever the
+# algorithm; a warp instruction is 32 lanes of an FMA (2 flop) to it.
+WEIGHTS_FP64_INSTRUCTIONS = 2.18e8 / 40962
 
 
 def weights_flops(m):
@@ -334,6 +340,23 @@ def json_safe(o):
     return o
 
 
+# The line on stdout keeps these of the full record, so that it stays short enough to be read from the end of a log.
+CONTRACT_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                 "vs_baseline", "dtype", "data", "config", "step_latency_ms", "fp64", "clocks", "e2e", "gpu_launches",
+                 "roofline")
+
+
+def contract_line(record):
+    """The record's contract keys and the headline of its legs."""
+    line = {k: record[k] for k in CONTRACT_KEYS}
+    direct = record["mixed_vs_fp64_at_equal_l2"]["direct"]
+    line["l2_vs_exact"] = {k: direct[k + "_l2_vs_exact"] for k in ("mixed", "fp64")}
+    line["center_value"] = record["center_stencils"]["mixed"]["value"]
+    cpu = record["cpu_baseline"]
+    line["cpu_baseline"] = {k: cpu[k] for k in ("value", "unit", "cores", "kind")} if cpu else None
+    return line
+
+
 def finite_or_none(v):
     v = float(v)
     return v if np.isfinite(v) else None
@@ -488,7 +511,7 @@ def bench_global_eval(rbfsl, torch, stream, flush, K=10):
             "fp32_cuda_cores": {"us": 1e3 * t32, "useful_tflops": flop / (t32 * 1e-3) / 1e12,
                                 "max_err_vs_fp64_rel_to_max": float((o32.double() - o64).abs().max()) / scale},
             "fp64": {"us": 1e3 * t64, "useful_tflops": flop / (t64 * 1e-3) / 1e12},
-            "fp32_pairs": {"kernel": "phi_pairs_kernel + cardinal_apply_pair_kernel (FP64 kernel values, pair sums)",
+            "fp32_pairs": {"kernel": "split_gemm_kernel<SrcPhi> (FP64 kernel values, digit products) + split_reduce<float2>",
                            "us": 1e3 * t_pr, "useful_tflops": flop / (t_pr * 1e-3) / 1e12,
                            "max_err_vs_fp64_rel_to_max": float(((o_pr[..., 0].double() + o_pr[..., 1].double())
                                                                 - o64).abs().max()) / scale}}
@@ -1114,9 +1137,7 @@ def main():
     # FP64 FMA throughput measured in this run (the weights kernel is timed alone: a burst rate)
     with ClockSampler(local) as clk_peak:
         fp64_peak = rbfsl.rbfsl_fp64_fma_rate(1 << 15, stream=stream)
-    w_flops = N * weights_flops(m)
-    w_tflops = w_flops / (w_ms * 1e-3) / 1e12
-    wk_tflops = N * weights_kernel_flops(m) / (w_ms * 1e-3) / 1e12
+    w_tflops = N * WEIGHTS_FP64_INSTRUCTIONS * 64 / (w_ms * 1e-3) / 1e12
     g_bytes = N * n * (8 + 4) + N * T * 8 * 2  # FP32-pair weights and field
     g_gbs = g_bytes / (g_ms * 1e-3) / 1e9
     line = {
@@ -1141,19 +1162,16 @@ def main():
         "clocks": clk.summary(),
         "e2e": e2e,
         "gpu_launches": 5 * args.steps,
-        "roofline": {"bound": "alu", "kernel": "weights_kernel<4, 4, float2> (reduced LDL^T, products as FP16 digit products, m = 109)",
+        "roofline": {"bound": "alu", "kernel": "weights_kernel<4, 4, float2> (reduced L D L^T, m = 109)",
                      "achieved": w_tflops, "peak": fp64_peak, "unit": "TFLOP/s",
-                     "frac": w_tflops / fp64_peak, "traffic": WEIGHTS_DRAM_BYTES,
-                     "traffic_unit": "bytes per launch (ncu dram__bytes_read + _write of this kernel version, "
-                                     "full launch; null: not captured for this version)",
-                     "peak_source": "measured in this run: rbfsl_fp64_fma_rate (dependent FMA chains, all SMs)",
-                     "peak_clocks": clk_peak.summary(),
-                     "peak_derived": FP64_PEAK_TFLOPS,
-                     "frac_of_derived": w_tflops / FP64_PEAK_TFLOPS,
-                     "flops_per_unit": "(2/3) m^3 + 2 m^2 per point (one saddle-point solve, elimination's count)",
-                     "kernel_flops_per_unit": "(1/3) m^3 + 2 m^2 (a symmetric solve; two products run on the tensor cores, so the fraction may pass 1)",
-                     "kernel_achieved": wk_tflops, "kernel_frac": wk_tflops / fp64_peak,
-                     "ms_per_launch": w_ms},
+                     "frac": w_tflops / fp64_peak, "traffic": WEIGHTS_DRAM_BYTES, "traffic_unit": "bytes per launch (ncu)",
+                     "flops_per_unit": "64 per FP64 warp instruction, %.0f of them a point (ncu)" % WEIGHTS_FP64_INSTRUCTIONS,
+                     "peak_source": "rbfsl_fp64_fma_rate, this run", "ms_per_launch": w_ms},
+        "roofline_peak": {"clocks": clk_peak.summary(), "derived": FP64_PEAK_TFLOPS},
+        # the FP64 work that other solutions of the same systems would need in this time: elimination, and an
+        # L D L^T of the whole system
+        "weights_equivalent_tflops": {"elimination": N * weights_flops(m) / (w_ms * 1e-3) / 1e12,
+                                      "ldl": N * weights_kernel_flops(m) / (w_ms * 1e-3) / 1e12},
         "roofline_gather": {"bound": "hbm", "kernel": "gather_dot_vec_kernel<float, float4>",
                             "workload": "N=655362 Morton-ordered nodes, n=84, T=16, FP32 difference form",
                             "achieved": wq["f32"]["achieved_gbs"], "peak": pk.get("hbm_gbs"), "unit": "GB/s",
@@ -1167,7 +1185,13 @@ def main():
         "cpu_baseline": cpu,
     }
     if rank == 0:
-        print(json.dumps(json_safe(line), allow_nan=False), flush=True)
+        record = json_safe(line)
+        if args.record:
+            with open(args.record, "w") as f:
+                json.dump(record, f, allow_nan=False)
+        else:
+            print(json.dumps(record, allow_nan=False), file=sys.stderr, flush=True)
+        print(json.dumps(contract_line(record), allow_nan=False), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
 
