@@ -12,7 +12,9 @@
 // Blocks of four warps: 16 rows x 32 columns per warp, as 2 x 2 warps (32 rows x 64 columns) or,
 // for up to 32 columns, 4 x 1 (64 rows). Bound: the tensor cores' FP16 rate, 43 digit products per
 // useful one (43 N^2 T / 304 TMAC/s: 0.95 ms at N = 10,242, T = 64, where the FP64 pipe takes
-// 10.7 ms), for few columns the digit extraction and the A stream.
+// 10.7 ms; the cardinal product 1.9 ms there, tensor pipe 45% busy, 612 us at N = 5,003, the rest digit extraction
+// between a chunk's barriers); for few columns the digit extraction and the A stream; in the evaluation the FP64
+// kernel values (5.4 ms for the same sizes with the Gaussian, 18.0 in FP64; FP64 pipe 78% busy).
 #include <algorithm>
 #include <type_traits>
 
@@ -301,12 +303,12 @@ int launch_gemm(const Src &A, int64_t M, int64_t K, const V *x, int T, int Tp, c
 
 // ---- triangular solves with diagonal blocks of 128 rows
 constexpr int kB = 64;  // inverted triangular blocks (two to a diagonal block)
-// Condition of a block above which its inverse's product is corrected (solve_diag). Below it the product's
-// residual, relative to |T| |x|, is within four times substitution's (blocks of Gaussian and IMQ factors, N = 1,000 to
-// 4,999; from 64 on up to a hundred times); a correction of every block made the step of N = 4,999, T = 9
-// 2.21 instead of 1.89 ms and that of N = 10,242, T = 64 4.67 instead of 3.94, though nine tenths of their
-// blocks lie below 16.
-constexpr double kSolveCond = 16.0;
+// Condition of a block above which its inverse's product is corrected (solve_diag). Residuals of whole solves against
+// plain substitution's, Gaussian and IMQ factors of 1,000 to 10,242 nodes from well conditioned to flat, sixteen
+// fields each: up to 64 the same as with every block corrected (largest 1.9 times, root mean square 1.1), from 256 on 3.0
+// and 1.2, from 1,024 2.9 and 2.2, without corrections 202 and 111. A solve at N = 1,000, T = 16: 469 us with every
+// block corrected, 415 (from 16 on), 368 (64), 355 without; at N = 10,242, most blocks below 64, 3.17 ms, 2.71, 2.58, 2.51.
+constexpr double kSolveCond = 64.0;
 
 // Programmatic dependent launch: the next kernel of the stream may start (its prologue runs beside this
 // kernel), and wait until every kernel before this one is complete. What an earlier kernel of the chain
@@ -510,7 +512,7 @@ __global__ void __launch_bounds__(256, 1) solve_diag(const double *__restrict__ 
 // waiting for the one before: few rows a block, the factor's digits formed beside the kernel before, and,
 // where that leaves SMs idle, the inner dimension split over the warps (launch_update). N = 4,999, T = 9, a step (80 links, evaluation
 // 0.83 ms): 64-row blocks with a warp's whole inner dimension, each link after the one before 3.30 ms, now
-// 1.88; N = 10,242, T = 64 (160 links) 7.37 ms, with prologues beside the link before 6.89, now 4.02 (4.20 before
+// 1.85; N = 10,242, T = 64 (160 links) 7.37 ms, with prologues beside the link before 6.89, now 3.99 (4.20 before
 // solve_diag left out the triangles' empty tiles).
 constexpr int64_t kUpdateBlocks = 4 * 152;
 
