@@ -136,10 +136,12 @@ int rbfsl_knn_query(const rbfsl_knn_index *index, const double *q, int64_t Nq, i
  *   [[A, P], [P^T, 0]] w~ = [phi(|p_i - x_Sj|)_j ; Y(p_i)],   w[i, :] = w~[0:n],
  * A_jk = phi(|x_Sj - x_Sk|), P_jc = Y_c(x_Sj), Y = real orthonormal spherical harmonics
  * of degree <= ell. Then the interpolant at p_i is sum_j w_ij f_Sj (the system is
- * symmetric). Solved by a symmetric indefinite L D L^T factorisation with Bunch-Kaufman
- * pivoting (1 x 1 and 2 x 2 pivots; blocked: the trailing update once per panel of four pivot
- * columns), one warp per point for small systems, four warps for larger ones; the result does
- * not depend on that choice.
+ * symmetric). Where (p - 1) / 2 <= ell for r^p and n > (ell+1)^2, the harmonics are eliminated first (LU with
+ * partial pivoting of P) and the reduced matrix, which is definite then, is factorised as L D L^T without
+ * interchanges; its two large products run as digit products on the tensor cores from 16 harmonics on. Other systems,
+ * and points whose reduced matrix breaks down, by a symmetric indefinite L D L^T with Bunch-Kaufman pivoting (1 x
+ * 1 and 2 x 2 pivots, panels of four columns). One, two or four warps per point by the system's size; the result
+ * does not depend on that choice.
  *   x: device N x 3; idx: device Nq x n; p: device Nq x 3; w: device Nq x n of w_dtype
  *   (RBFSL_F64, RBFSL_F32 or RBFSL_F32X2: FP64 solve, result rounded or split into an FP32
  *   pair). status: device Nq or NULL
@@ -276,12 +278,11 @@ int rbfsl_pu_apply(rbfsl_pu *pu, const double *q, int T, const double *p, int64_
  * up (out is then unspecified), otherwise left unchanged. Asynchronous on `stream`.
  * Errors: EINVAL (sizes, kernel, dtype, workspace too small or misaligned), ECUDA. */
 /* Global-interpolant evaluation to FP64 accuracy without FP64 products: Phi(p, x) formed in
- * FP64 (the kernel and distance arithmetic of rbfsl_global_eval) and stored as FP32 pairs, the
- * coefficients split into pairs, then out = Phi c by FP32-pair arithmetic (the product of
- * rbfsl_cardinal_apply): ~2^-48 relative per term. c: device N x T FP64; out: device Nq x T
- * FP32 pairs (Nq x T x 2 floats). workspace: device, 256-byte aligned, at least
- * rbfsl_global_eval_pairs_workspace_bytes(Nq, N, T) (Nq x N x 8 bytes for Phi, the split
- * coefficients and the product's split-K partials); owned by the caller, not shared between
+ * FP64 (the kernel and distance arithmetic of rbfsl_global_eval) on the way, out = Phi c as exact digit products
+ * on the tensor cores whose chunks of 128 nodes are added in FP64, the sums split into FP32 pairs. c: device N x T
+ * FP64; out: device Nq x T FP32 pairs (Nq x T x 2 floats). workspace: device, 256-byte aligned, at least
+ * rbfsl_global_eval_pairs_workspace_bytes(Nq, N, T) (the digits of c, 8 bytes a value, and partial
+ * sums of up to 32 times the result in FP64); owned by the caller, not shared between
  * calls that overlap on the GPU. Asynchronous on `stream`. Errors: EINVAL, ECUDA. */
 size_t rbfsl_global_eval_pairs_workspace_bytes(int64_t Nq, int64_t N, int T);
 int rbfsl_global_eval_pairs(const double *p, int64_t Nq, const double *x, int64_t N, int kernel,
@@ -303,21 +304,21 @@ int rbfsl_global_eval_tc(const double *p, int64_t Nq, const double *x, int64_t N
  *   symmetric, so E^T = A_X^-1 Phi(P, X)^T is solved with it in blocks of points).
  *   x: device N x 3; p: device Nq x 3. E: device Nq x N row-major, e_dtype RBFSL_F64 (doubles)
  *   or RBFSL_F32X2 (FP32 pairs hi = fl32(e), lo = fl32(e - hi); Nq x N x 2 floats), computed in
- *   FP64 either way. Allocates and frees 2 N min(Nq, 512) doubles of device scratch and
- *   synchronises `stream`. Errors: EINVAL (sizes, kernel, dtype, null pointers), ENOMEM, ECUDA. */
+ *   FP64 either way. Allocates and frees 2 N min(Nq, 512) doubles of device scratch and rbfsl_global_solve's
+ *   scratch for 512 fields (1.5 kB a row), and synchronises `stream`. Errors: EINVAL (sizes, kernel, dtype, null pointers), ENOMEM, ECUDA. */
 int rbfsl_global_cardinal(const double *LU, const int32_t *perm, const double *x, int64_t N,
                           int kernel, double eps, const double *p, int64_t Nq, void *E,
                           int e_dtype, void *stream);
 
 /* q_out = E q for a cardinal matrix E (Nq x N) and T fields q (N x T), row-major:
  *   q_out[i][t] = sum_j E[i][j] q[j][t].
- * dtype RBFSL_F64: E, q, q_out doubles, FP64 arithmetic. RBFSL_F32X2: FP32 pairs, each term
- * formed in pair arithmetic with FP32 operations only (relative rounding ~2^-48 per term; the
- * cardinal values are O(1), so there is no cancellation to amplify it).
- * The sum over j is split into ranges so that the grid covers the device; the partial sums go
- * to `workspace` (at least rbfsl_cardinal_apply_workspace_bytes(Nq, N, T) bytes on the calling
- * device, 0 when no split is needed; the caller owns it and must not share it between calls that
- * overlap on the GPU) and are added in a fixed order, so the result is deterministic for a given
+ * dtype RBFSL_F64: E, q, q_out doubles. RBFSL_F32X2: FP32 pairs. Both as exact digit products on the tensor cores,
+ * to FP64 accuracy: a chunk of 128 terms is off by less than 2^-52 of its row's times its column's largest entry,
+ * the chunks are added in FP64.
+ * The sum over j is split into ranges so that the grid covers the device; q's digits (8 bytes a value) and the partial
+ * sums go to `workspace` (at least rbfsl_cardinal_apply_workspace_bytes(Nq, N, T) bytes on the calling
+ * device, 0 for Nq = 0 only; the caller owns it and must not share it between calls that
+ * overlap on the GPU); the sums are added in a fixed order, so the result is deterministic for a given
  * device. q_out may not alias q. Asynchronous on `stream`.
  * Errors: EINVAL (sizes, dtype, null pointers, workspace too small), ECUDA. */
 size_t rbfsl_cardinal_apply_workspace_bytes(int64_t Nq, int64_t N, int T);
@@ -375,7 +376,7 @@ int rbfsl_set_integrator(rbfsl_ctx *ctx, int order);
  * A_X^-1 q and the evaluation at the departure points (Sec. 3.3). RBFSL_GLOBAL_CARDINAL: the
  * departure points are traced once and E = Phi(Xi, X) A_X^-1 is formed at preparation
  * (rbfsl_global_cardinal; A_X's factor is freed afterwards), each step is q <- E q
- * (rbfsl_cardinal_apply: FP64, or FP32-pair arithmetic in RBFSL_MIXED). Valid for a steady
+ * (rbfsl_cardinal_apply: FP64, or FP32 pairs in RBFSL_MIXED). Valid for a steady
  * velocity only (RBFSL_VEL_RIGID; the first step returns EINVAL otherwise). Invalidates
  * prepared state, as do set_dt and set_integrator while the cardinal form is selected (E
  * depends on the departure points). Errors: EINVAL. */
@@ -384,10 +385,10 @@ int rbfsl_set_global_form(rbfsl_ctx *ctx, int form);
 /* Evaluation arithmetic of the RBFSL_GLOBAL_SOLVE step in RBFSL_MIXED (the solve is FP64 in
  * both). RBFSL_GLOBAL_EVAL_TC (default): split-TF32 products on the tensor cores
  * (rbfsl_global_eval_tc; fastest, ~2^-22 relative). RBFSL_GLOBAL_EVAL_PAIRS: kernel values in
- * FP64, the sum Phi(Xi, X) C in FP32 pairs (rbfsl_global_eval_pairs; ~2^-48 relative, an N x N
- * pair workspace). Where the interpolation matrix is ill-conditioned the iteration feeds the
- * evaluation's rounding back through the next solve, so neither matches FP64 there (at Gaussian
- * eps = 9 on 10,242 nodes both diverge while FP64 does not); the cardinal form does.
+ * FP64, the sum Phi(Xi, X) C to FP64 accuracy, rounded to FP32 pairs (rbfsl_global_eval_pairs). Where the
+ * interpolation matrix is ill-conditioned the iteration feeds the field's rounding back through the next
+ * solve: at Gaussian eps = 9 on 10,242 nodes, 200 steps, the tensor-core form diverges, the pairs end 2% above FP64's
+ * error; the cardinal form matches FP64.
  * Invalidates prepared state. Errors: EINVAL. */
 enum { RBFSL_GLOBAL_EVAL_PAIRS = 0, RBFSL_GLOBAL_EVAL_TC = 1 };
 int rbfsl_set_global_eval(rbfsl_ctx *ctx, int kind);

@@ -283,7 +283,7 @@ def rbfsl_global_eval(p, x, kernel, eps, c, out, stream=None):
 
 
 class PUPatches:
-    """RBF-PU patches with their LU factors (rbfsl_pu_create / rbfsl_pu_destroy)."""
+    """RBF-PU patches with their factors (rbfsl_pu_create / rbfsl_pu_destroy)."""
 
     def __init__(self, x, centers, radius, ell, kernel, kparam, stream=None):
         self._h = ctypes.c_void_p()
@@ -491,7 +491,7 @@ def rbfsl_global_eval_tc(p, x, kernel, eps, c, out, workspace=None, status=None,
 
 
 def rbfsl_global_eval_pairs(p, x, kernel, eps, c, out, workspace=None, stream=None):
-    """FP64-accurate evaluation in FP32-pair arithmetic; c: FP64 N x T; out: float32 Nq x T x 2;
+    """FP64-accurate evaluation, the sums as FP32 pairs; c: FP64 N x T; out: float32 Nq x T x 2;
     workspace: a uint8 device tensor (allocated here when None, 256-byte aligned)."""
     import torch
     T = c.shape[1] if c.dim() == 2 else 1
@@ -521,7 +521,7 @@ def rbfsl_global_cardinal(LU, perm, x, kernel, eps, p, E, stream=None):
 
 
 def rbfsl_cardinal_apply(E, q, out, workspace=None, stream=None):
-    """out = E q (FP64, or FP32-pair arithmetic for pair tensors); workspace: a uint8 device
+    """out = E q (FP64, or FP32 pairs for pair tensors); workspace: a uint8 device
     tensor (allocated here when None), returned for reuse."""
     import torch
     code = _f64_or_pairs(E)
