@@ -452,13 +452,23 @@ int global_solve_plain(const double *LU, const int32_t *perm, int64_t N, const d
 
 namespace {
 
-// Stream-ordered scratch of one call; null where none can be had: under capture (a graph would keep
-// the allocation) or out of memory. The caller then takes the form without scratch.
+// While another stream is captured in the global mode (or this thread captures one), an allocation counts as
+// potentially unsafe and would end that capture; one on a stream that is not captured is not, so the
+// thread says so for its duration.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Stream-ordered scratch of one call; null where none can be had: under capture of its stream (a graph would
+// keep the allocation) or out of memory. The caller then takes the form without scratch.
 struct Scratch {
     void *p = nullptr;
     cudaStream_t s;
     Scratch(size_t bytes, cudaStream_t st) : s(st) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        RelaxedCapture relaxed;
         if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
             cudaMallocAsync(&p, bytes, s) != cudaSuccess) {
             cudaGetLastError();
@@ -466,6 +476,7 @@ struct Scratch {
         }
     }
     ~Scratch() {
+        RelaxedCapture relaxed;
         if (p) cudaFreeAsync(p, s);
     }
     Scratch(const Scratch &) = delete;
